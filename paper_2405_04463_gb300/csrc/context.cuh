@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "gemm_ts.cuh"
 
 namespace ipc {
 const char* thread_last_error();
@@ -84,12 +85,6 @@ int ring_gemm_compare_tc(uint32_t segments, const int8_t* const x_lo[6], const i
 int or_join_parts_launch(const uint32_t* parts, size_t ld_parts, uint32_t n_cols, size_t n_rows, uint64_t row0,
                          const uint32_t* col_tags, const uint64_t seeds[3], uint32_t* roots, size_t ld_roots,
                          cudaStream_t st);
-int ring_gemm_tc_variant(uint32_t tile_cols, uint32_t segments, const int8_t* const x_lo[2],
-                         const int8_t* const x_hi[2], size_t x_rows, const uint16_t* b_lo, const uint16_t* b_hi,
-                         uint32_t n_cols, uint32_t n_pad, uint32_t l, const uint32_t* col_tags, uint64_t seed_own,
-                         uint64_t seed_prev, uint32_t vec, uint16_t* z, size_t ldz, uint64_t row0,
-                         const uint32_t* col_tiles, const uint32_t* n_col_list, cudaStream_t stream);
-
 // Serving hooks defined in serve.cu. serve_fetch_shares and serve_release return IPC_ENOTFOUND
 // for ids that are not serving requests.
 int serve_fetch_shares(ipc_ctx* c, uint64_t id, uint8_t* out, size_t n, int timeout_ms);

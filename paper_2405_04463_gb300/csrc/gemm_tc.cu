@@ -1,7 +1,9 @@
-// A3 on the 5th-generation tensor cores: tcgen05.mma (kind::f16) with fp16 operands carrying the
-// balanced int8 limbs, fp32 accumulators in tensor memory.
+// The fused chunk step (ipc_config.fused): the six ring GEMMs of a chunk (A3) tile by tile on the
+// 5th-generation tensor cores, each tile followed by its comparison phase (A4-A8), in one launch. Its
+// GEMM keeps both operands in shared memory and accumulators in tensor memory; the unfused steps use the
+// form with the database operand in tensor memory (gemm_ts.cu), which leaves no room for the comparison.
 //
-// The ring product is the same three limb products as the int8 paths (Sec. 6.1):
+// The ring product is three limb products (Sec. 6.1):
 //     z = L + 256 C + r  (mod 2^16),  L = sum lo*lo',  C = sum (lo*hi' + hi*lo').
 // sm_103a has no integer tcgen05 kind, but the arithmetic stays exact on the f16 kind:
 //   * every limb is an integer in [-128, 127], exactly an fp16 value;
@@ -25,7 +27,7 @@
 // ahead, and widens them into the W ring up to WS - 1 k-blocks ahead of the MMAs; the two warps
 // never wait for each other.
 //
-// Roles (one CTA per tile of 128 database rows x TN query columns, 12 warps):
+// Roles (persistent, one CTA per SM, tiles of 128 database rows x TN query columns, 12 warps):
 //   warp 0 lane 0  query producer: per k-block of 32 elements, the two query tiles.
 //   warps 10-11    raw copies and widening of the lo (warp 10) and hi (warp 11) limb plane.
 //   warp 1 lane 0  MMA issuer: per chunk of four k-blocks, the C products (2 MMAs of 128xTNx16
@@ -38,7 +40,6 @@
 //                  drained while the chunk's last L products run, L while the next chunk's first
 //                  C products run, so the tensor pipe does not wait for the drain.
 // TMEM: L in columns [0, TN), C in [TN, 2 TN).
-// Tile widths TN = 256 (the fixed-shape launch) and 128; see gemm_tc_kernel for the list mode.
 // Every wait is bounded (2 s, or sooner once another role has failed); a failed CTA raises the
 // status word, lets its copies and MMAs finish, frees its tensor memory and stores nothing.
 #include "compare.cuh"
@@ -65,11 +66,10 @@ constexpr int WIDEN_WARP0 = 10, WIDEN_THREADS = 2 * 32;
 constexpr int NUM_BARS = 2 * QS + WS + 2 * RS + 6;
 constexpr uint32_t MAGIC = 0x4B400000u;  // fp32 bits of 1.5 * 2^23
 
-// Tile shape: TN query columns per tile (MMA N = 256 or 128). Shared memory, 1024-byte aligned:
+// Tile shape: TN query columns per tile (MMA N). Shared memory, 1024-byte aligned:
 // the Q ring (first: the epilogue stages z there), the W ring, the R ring, the barriers.
 template <int TN>
 struct Shape {
-  static_assert(TN == 256 || TN == 128, "tile width");
   static constexpr int B_BYTES = TN * KB * 2;
   static constexpr int Q_STAGE = 2 * B_BYTES, W_STAGE = 2 * A_BYTES, R_STAGE = 2 * A_RAW;
   static constexpr int W_OFF = QS * Q_STAGE, R_OFF = W_OFF + WS * W_STAGE, BAR_OFF = R_OFF + RS * R_STAGE;
@@ -94,12 +94,7 @@ struct TcParams {
   uint32_t kb_total;  // K / KB (K = 2l, or l for Galois-ring shares)
   uint32_t kb_half;   // l / KB: k-blocks below it read the first database plane pair
   uint32_t n_row_tiles;
-  const uint32_t* col_tiles;   // list mode: the column tiles to compute (device)
-  const uint32_t* n_col_list;  // list mode: their count (device), read when the kernel starts
   const uint32_t* col_tags;
-  uint64_t seed_own, seed_prev;
-  uint32_t vec;
-  uint16_t* z;
   uint64_t ldz;
   uint64_t row0;
   uint32_t* status;
@@ -126,17 +121,8 @@ struct FuseParams {
   uint32_t* part_roots;    // [3][n_cols][ld_parts]: OR root of (column, row tile) of the chunk
   uint64_t ld_parts;
 };
-// The six tensor maps of a one-pass launch (kernel parameters).
-struct MapRefs {
-  const CUtensorMap *b_lo, *b_hi, *a0_lo, *a0_hi, *a1_lo, *a1_hi;
-};
 constexpr uint32_t FUSE_LOG2_BLOCK = 5;  // 1,024-row OR blocks: 8 row tiles of 128 rows
 
-// Without a list (LIST false) the grid is (column tiles, row tiles), one tile per CTA. With a list,
-// gridDim.x persistent CTAs walk items w = blockIdx.x + i * gridDim.x: column tile
-// list[w % n_ct], row tile w / n_ct; k-block and chunk counters run on across items, and the
-// query producer starts an item's copies once the previous item's epilogue has left the Q ring
-// (the raw and widened rings run on into the next item meanwhile).
 // bar.sync over n threads that also returns, to every one of them, whether any had pred set.
 __device__ __forceinline__ bool named_sync_or(uint32_t id, uint32_t n, bool pred) {
   uint32_t r;
@@ -176,49 +162,32 @@ __device__ __noinline__ void fused_part_compare(const TcParams& p, const FusePar
   fp.part_roots[2 * plane + at] = root.c2;
 }
 
-template <int TN, bool LIST, bool FUSE>
-__device__ __forceinline__ void gemm_tc_body(const MapRefs& mr, const FuseMaps* fm, const TcParams& p,
-                                             const FuseParams& fp) {
-  static_assert(!(LIST && FUSE), "the fused form walks the fixed shape");
-  constexpr bool PERSIST = LIST || FUSE;
+template <int TN>
+__device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams& p, const FuseParams& fp) {
   using S = Shape<TN>;
   constexpr int B_BYTES = S::B_BYTES;
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ uint32_t s_abort;
-  uint32_t n_ct = 0, my_items = 1;
-  if (LIST) {
-    n_ct = *p.n_col_list;
-    const uint32_t n_items = n_ct * p.n_row_tiles;
-    my_items = n_items > blockIdx.x ? (n_items - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-    if (my_items == 0) return;  // uniform for the CTA, before any barrier or allocation
-  }
-  if (FUSE) {
-    // items: the six passes of each of this CTA's tiles, tile after tile
-    n_ct = fp.n_ct;
-    const uint32_t n_tiles = n_ct * p.n_row_tiles;
-    const uint32_t my_tiles = n_tiles > blockIdx.x ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-    if (my_tiles == 0) return;
-    my_items = my_tiles * NPASS;
-  }
-  // Tiles are taken in linear order (blocks are dispatched in blockIdx order; a persistent CTA
-  // takes items blockIdx.x + i gridDim.x). The order walks bands of up to kBand column tiles,
+  // items: the six passes of each of this CTA's tiles, tile after tile
+  const uint32_t n_ct = fp.n_ct, n_tiles = n_ct * p.n_row_tiles;
+  const uint32_t my_tiles = n_tiles > blockIdx.x ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+  if (my_tiles == 0) return;  // uniform for the CTA, before any barrier or allocation
+  const uint32_t my_items = my_tiles * NPASS;
+  // A CTA takes tiles blockIdx.x + i gridDim.x of a linear order that walks bands of up to kBand column tiles,
   // all row tiles of a band before the next, so that the tiles in flight at once (one CTA per
   // SM) cover about 19 row tiles x 8 column tiles: each database tile is read by the band's
   // CTAs together and the band's query tiles stay in L2 while the rows stream past (with many
   // query columns the whole query operand is several times the L2).
   constexpr uint32_t kBand = 8;
   auto coords = [&](uint32_t i, uint32_t& q0, uint32_t& d0) {
-    const uint32_t n_cols_t = PERSIST ? n_ct : gridDim.x;
-    const uint32_t n_rt = PERSIST ? p.n_row_tiles : gridDim.y;
-    const uint32_t lin = FUSE   ? blockIdx.x + (i / NPASS) * gridDim.x
-                         : LIST ? blockIdx.x + i * gridDim.x
-                                : blockIdx.x + gridDim.x * blockIdx.y;
+    const uint32_t n_rt = p.n_row_tiles;
+    const uint32_t lin = blockIdx.x + (i / NPASS) * gridDim.x;
     const uint32_t band = lin / (kBand * n_rt), c0 = band * kBand;
-    const uint32_t width = n_cols_t - c0 < kBand ? n_cols_t - c0 : kBand;
+    const uint32_t width = n_ct - c0 < kBand ? n_ct - c0 : kBand;
     const uint32_t in_band = lin - band * kBand * n_rt;
     const uint32_t ct = c0 + in_band % width;
-    q0 = (LIST ? p.col_tiles[ct] : ct) * TN;
+    q0 = ct * TN;
     d0 = (in_band / width) * TM;
   };
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -275,8 +244,8 @@ __device__ __forceinline__ void gemm_tc_body(const MapRefs& mr, const FuseMaps* 
             break;
           }
           const uint32_t full = q_full + 8 * s, base = qring + s * S::Q_STAGE;
-          const CUtensorMap* mlo = FUSE ? &fm->q[i % NPASS][0] : mr.b_lo;
-          const CUtensorMap* mhi = FUSE ? &fm->q[i % NPASS][1] : mr.b_hi;
+          const CUtensorMap* mlo = &fm.q[i % NPASS][0];
+          const CUtensorMap* mhi = &fm.q[i % NPASS][1];
           mbar_expect_tx(full, 2 * B_BYTES);
           tma_load(base, mlo, static_cast<int32_t>(kb * KB), static_cast<int32_t>(q0), full);
           tma_load(base + B_BYTES, mhi, static_cast<int32_t>(kb * KB), static_cast<int32_t>(q0), full);
@@ -358,17 +327,11 @@ __device__ __forceinline__ void gemm_tc_body(const MapRefs& mr, const FuseMaps* 
     // k-block G + RS into raw stage G % RS once the warp has read k-block G from it.
     const uint32_t pl = static_cast<uint32_t>(warp - WIDEN_WARP0);  // 0: lo limbs, 1: hi limbs
     const uint32_t rf = r_full + 8 * RS * pl;
-    // the database planes of item i's two K segments: components ps / 2 and ps / 2 - 1 of the
-    // pass's vector in the fused form
+    // the database planes of item i's two K segments: components ps / 2 and ps / 2 - 1 of the pass's vector
     auto seg_maps = [&](uint32_t i, const CUtensorMap*& m0, const CUtensorMap*& m1) {
-      if (FUSE) {
-        const uint32_t ps = i % NPASS, party = ps >> 1, vec = ps & 1u;
-        m0 = &fm->x[2 * party + vec][pl];
-        m1 = &fm->x[2 * ((party + 2) % 3) + vec][pl];
-      } else {
-        m0 = pl ? mr.a0_hi : mr.a0_lo;
-        m1 = pl ? mr.a1_hi : mr.a1_lo;
-      }
+      const uint32_t ps = i % NPASS, party = ps >> 1, vec = ps & 1u;
+      m0 = &fm.x[2 * party + vec][pl];
+      m1 = &fm.x[2 * ((party + 2) % 3) + vec][pl];
     };
     const CUtensorMap *map0, *map1;
     // the next raw copy (lane 0): k-block li_kb of item li, whose row offset li_d0 and tensor
@@ -485,11 +448,9 @@ __device__ __forceinline__ void gemm_tc_body(const MapRefs& mr, const FuseMaps* 
       if (named_sync_or(1, DRAIN_THREADS, *abort != 0)) break;
       uint32_t q0, d0;
       coords(i, q0, d0);
-      const uint32_t ps = FUSE ? i % NPASS : 0u, party = ps >> 1;
-      const uint64_t seed_own = FUSE ? fp.seeds[party] : p.seed_own;
-      const uint64_t seed_prev = FUSE ? fp.seeds[(party + 2) % 3] : p.seed_prev;
-      const uint32_t vec = FUSE ? (ps & 1u) : p.vec;
-      uint16_t* const zout = FUSE ? fp.z[ps] : p.z;
+      const uint32_t ps = i % NPASS, party = ps >> 1, vec = ps & 1u;
+      const uint64_t seed_own = fp.seeds[party], seed_prev = fp.seeds[(party + 2) % 3];
+      uint16_t* const zout = fp.z[ps];
       uint16_t* zs = reinterpret_cast<uint16_t*>(smem);  // [TN][TM]
       const uint32_t row = 32 * q + lane;
 #pragma unroll
@@ -518,16 +479,13 @@ __device__ __forceinline__ void gemm_tc_body(const MapRefs& mr, const FuseMaps* 
                                    add2(acc.w, fo.w, fq.w));
         uint16_t* dst = zout + static_cast<uint64_t>(col) * p.ldz + r0;
         if (r0 + 8 <= p.x_rows) {
-          if (FUSE)
-            *reinterpret_cast<uint4*>(dst) = v;  // kept in L2: this CTA reads it back after the tile's last pass
-          else
-            __stcs(reinterpret_cast<uint4*>(dst), v);  // streamed: z is read by a later kernel, not from L2
+          *reinterpret_cast<uint4*>(dst) = v;  // kept in L2: this CTA reads it back after the tile's last pass
         } else {
           const uint32_t w[4] = {v.x, v.y, v.z, v.w};
           for (uint32_t e = 0; e < p.x_rows - r0; ++e) dst[e] = static_cast<uint16_t>(w[e >> 1] >> (16 * (e & 1)));
         }
       }
-      if (FUSE && ps == NPASS - 1) {
+      if (ps == NPASS - 1) {
         // ---- A4-A8 on the tile: its six z tiles are in global memory (L2), written by this
         // CTA's drainers; the barrier orders those stores before the reads below ----
         named_sync(1, DRAIN_THREADS);
@@ -546,88 +504,13 @@ __device__ __forceinline__ void gemm_tc_body(const MapRefs& mr, const FuseMaps* 
   }
 }
 
-template <int TN, bool LIST>
-__global__ void __launch_bounds__(THREADS, 1)
-    gemm_tc_kernel(const __grid_constant__ CUtensorMap tb_lo, const __grid_constant__ CUtensorMap tb_hi,
-                   const __grid_constant__ CUtensorMap ta0_lo, const __grid_constant__ CUtensorMap ta0_hi,
-                   const __grid_constant__ CUtensorMap ta1_lo, const __grid_constant__ CUtensorMap ta1_hi,
-                   const TcParams p) {
-  gemm_tc_body<TN, LIST, false>(MapRefs{&tb_lo, &tb_hi, &ta0_lo, &ta0_hi, &ta1_lo, &ta1_hi}, nullptr, p,
-                                FuseParams{});
-}
-
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_cmp_kernel(const __grid_constant__ FuseMaps fm, const __grid_constant__ TcParams p,
                     const __grid_constant__ FuseParams fp) {
-  gemm_tc_body<256, false, true>(MapRefs{}, &fm, p, fp);
-}
-
-template <int TN, bool LIST>
-int launch_tc(const CUtensorMap* m, const TcParams& p, dim3 grid, cudaStream_t stream) {
-  static PerDevice attr;
-  IPC_CUDA_TRY(attr.run([] {
-    return cudaFuncSetAttribute(gemm_tc_kernel<TN, LIST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                Shape<TN>::SMEM_BYTES);
-  }));
-  gemm_tc_kernel<TN, LIST><<<grid, THREADS, Shape<TN>::SMEM_BYTES, stream>>>(m[0], m[1], m[2], m[3], m[4], m[5], p);
-  IPC_CUDA_TRY(cudaGetLastError());
-  return IPC_OK;
+  gemm_tc_body<256>(fm, p, fp);
 }
 
 }  // namespace
-
-// tile_cols: 256 or 128 query columns per tile. With col_tiles set, only the listed tiles of
-// that width are computed (n_col_list, on the device, holds their count) by one persistent CTA
-// per SM; otherwise every tile of [0, n_cols), one CTA each. segments: 2 for K = 2l over the
-// planes [x_lo[0] | x_lo[1]] (replicated sharing), 1 for K = l over x_lo[0] alone (Galois-ring
-// Shamir shares; l a multiple of 256 so that L's 256-k drains tile K).
-int ring_gemm_tc_variant(uint32_t tile_cols, uint32_t segments, const int8_t* const x_lo[2],
-                         const int8_t* const x_hi[2], size_t x_rows, const uint16_t* b_lo, const uint16_t* b_hi,
-                         uint32_t n_cols, uint32_t n_pad, uint32_t l, const uint32_t* col_tags, uint64_t seed_own,
-                         uint64_t seed_prev, uint32_t vec, uint16_t* z, size_t ldz, uint64_t row0,
-                         const uint32_t* col_tiles, const uint32_t* n_col_list, cudaStream_t stream) {
-  if (tile_cols != 256 && tile_cols != 128) {
-    set_error("tcgen05 ring GEMM: tile width must be 128 or 256");
-    return IPC_EINVAL;
-  }
-  if (segments != 1 && segments != 2) {
-    set_error("tcgen05 ring GEMM: one or two K segments");
-    return IPC_EINVAL;
-  }
-  if ((segments * l) % (2 * KB_PER_CHUNK * KB) != 0) {
-    set_error("tcgen05 ring GEMM: K must be a multiple of 256");
-    return IPC_EINVAL;
-  }
-  CUtensorMap m[6];
-  int rc;
-  if ((rc = make_map_f16(&m[0], b_lo, static_cast<uint64_t>(segments) * l, n_pad, tile_cols)) ||
-      (rc = make_map_f16(&m[1], b_hi, static_cast<uint64_t>(segments) * l, n_pad, tile_cols)) ||
-      (rc = make_map_i8(&m[2], x_lo[0], l, x_rows, TM)) || (rc = make_map_i8(&m[3], x_hi[0], l, x_rows, TM)) ||
-      (rc = make_map_i8(&m[4], x_lo[1], l, x_rows, TM)) || (rc = make_map_i8(&m[5], x_hi[1], l, x_rows, TM)))
-    return rc;
-  TcParams p;
-  p.n_cols = n_cols;
-  p.x_rows = static_cast<uint32_t>(x_rows);
-  p.kb_total = segments * l / KB;
-  p.kb_half = l / KB;  // with one segment every k-block reads x_lo[0] / x_hi[0]
-  p.n_row_tiles = static_cast<uint32_t>((x_rows + TM - 1) / TM);
-  p.col_tiles = col_tiles;
-  p.n_col_list = n_col_list;
-  p.col_tags = col_tags;
-  p.seed_own = seed_own;
-  p.seed_prev = seed_prev;
-  p.vec = vec;
-  p.z = z;
-  p.ldz = ldz;
-  p.row0 = row0;
-  p.status = status_ptr();
-  if (col_tiles) {
-    const dim3 grid(static_cast<unsigned>(sm_count_current()));
-    return tile_cols == 256 ? launch_tc<256, true>(m, p, grid, stream) : launch_tc<128, true>(m, p, grid, stream);
-  }
-  const dim3 grid((n_cols + tile_cols - 1) / tile_cols, p.n_row_tiles);
-  return tile_cols == 256 ? launch_tc<256, false>(m, p, grid, stream) : launch_tc<128, false>(m, p, grid, stream);
-}
 
 // The fused chunk step: the six ring GEMMs of a chunk (replicated sharing, segments = 2: party i
 // reads components i and i - 1 of each vector; Galois-ring Shamir shares, segments = 1: party i
@@ -691,14 +574,6 @@ int ring_gemm_compare_tc(uint32_t segments, const int8_t* const x_lo[6], const i
   gemm_cmp_kernel<<<grid, THREADS, Shape<256>::SMEM_BYTES, stream>>>(fm, p, fp);
   IPC_CUDA_TRY(cudaGetLastError());
   return IPC_OK;
-}
-
-int ring_gemm_tc(const int8_t* const x_lo[2], const int8_t* const x_hi[2], size_t x_rows, const uint16_t* b_lo,
-                 const uint16_t* b_hi, uint32_t n_cols, uint32_t n_pad, uint32_t l, const uint32_t* col_tags,
-                 uint64_t seed_own, uint64_t seed_prev, uint32_t vec, uint16_t* z, size_t ldz, uint64_t row0,
-                 cudaStream_t stream) {
-  return ring_gemm_tc_variant(256, 2, x_lo, x_hi, x_rows, b_lo, b_hi, n_cols, n_pad, l, col_tags, seed_own,
-                              seed_prev, vec, z, ldz, row0, nullptr, nullptr, stream);
 }
 
 }  // namespace ipc

@@ -129,6 +129,8 @@ int batch_part(ipc_ctx* c, const uint16_t* const code[3], const uint16_t* const 
     zc[i] = bb.z + (static_cast<size_t>(0) * 3 + i) * N * ldz;
     zm[i] = bb.z + (static_cast<size_t>(1) * 3 + i) * N * ldz;
   }
+  const bool tensor = c->cfg.path == IPC_PATH_TC || c->cfg.path == IPC_PATH_TCG;
+  RingGemm gemms[RING_GEMM_PASSES];  // tcgen05 paths: the six GEMMs in one launch
   for (int i = 0; i < 3; ++i) {
     const int prev = (i + 2) % 3;
     for (int vec = 0; vec < 2; ++vec) {
@@ -136,21 +138,23 @@ int batch_part(ipc_ctx* c, const uint16_t* const code[3], const uint16_t* const 
       uint16_t* zo = vec == 0 ? zc[i] : zm[i];
       auto p16 = [](const uint8_t* p) { return reinterpret_cast<const uint16_t*>(p); };
       auto p8 = [](const uint8_t* p) { return reinterpret_cast<const int8_t*>(p); };
-      if (c->cfg.path == IPC_PATH_TCG) {
-        P_RC(ipc_prep_query_galois(y, P, &g, i, reinterpret_cast<uint16_t*>(bq(i, vec, 0)),
-                                   reinterpret_cast<uint16_t*>(bq(i, vec, 1)), n_pad, st));
-        const int8_t* xl[2] = {p8(pl(i, vec, 0)), p8(pl(i, vec, 0))};
-        const int8_t* xh[2] = {p8(pl(i, vec, 1)), p8(pl(i, vec, 1))};
-        P_RC(ring_gemm_tc_variant(256, 1, xl, xh, P, p16(bq(i, vec, 0)), p16(bq(i, vec, 1)), N, n_pad, l, bb.tags,
-                                  c->cfg.seeds[i], c->cfg.seeds[prev], static_cast<uint32_t>(vec), zo, ldz, 0,
-                                  nullptr, nullptr, st));
-      } else if (c->cfg.path == IPC_PATH_TC) {
-        P_RC(ipc_prep_query_f16(y, P, &g, i, reinterpret_cast<uint16_t*>(bq(i, vec, 0)),
-                                reinterpret_cast<uint16_t*>(bq(i, vec, 1)), n_pad, st));
-        const int8_t* xl[2] = {p8(pl(i, vec, 0)), p8(pl(prev, vec, 0))};
-        const int8_t* xh[2] = {p8(pl(i, vec, 1)), p8(pl(prev, vec, 1))};
-        P_RC(ipc_ring_gemm_tc(xl, xh, P, p16(bq(i, vec, 0)), p16(bq(i, vec, 1)), N, n_pad, l, bb.tags, c->cfg.seeds[i],
-                              c->cfg.seeds[prev], static_cast<uint32_t>(vec), zo, ldz, 0, st));
+      if (tensor) {
+        uint16_t* lo = reinterpret_cast<uint16_t*>(bq(i, vec, 0));
+        uint16_t* hi = reinterpret_cast<uint16_t*>(bq(i, vec, 1));
+        const int other = c->cfg.path == IPC_PATH_TCG ? i : prev;
+        if (other == i)
+          P_RC(ipc_prep_query_galois(y, P, &g, i, lo, hi, n_pad, st));
+        else
+          P_RC(ipc_prep_query_f16(y, P, &g, i, lo, hi, n_pad, st));
+        gemms[3 * vec + i] = RingGemm{{p8(pl(i, vec, 0)), p8(pl(other, vec, 0))},
+                                      {p8(pl(i, vec, 1)), p8(pl(other, vec, 1))},
+                                      other == i ? 1u : 2u,
+                                      p16(bq(i, vec, 0)),
+                                      p16(bq(i, vec, 1)),
+                                      c->cfg.seeds[i],
+                                      c->cfg.seeds[prev],
+                                      static_cast<uint32_t>(vec),
+                                      zo};
       } else {
         P_RC(ipc_prep_query(y, P, &g, i, reinterpret_cast<int8_t*>(bq(i, vec, 0)),
                             reinterpret_cast<int8_t*>(bq(i, vec, 1)), n_pad, st));
@@ -161,6 +165,7 @@ int batch_part(ipc_ctx* c, const uint16_t* const code[3], const uint16_t* const 
       }
     }
   }
+  if (tensor) P_RC(ring_gemm_ts(6, gemms, P, N, n_pad, l, bb.tags, ldz, 0, 0, nullptr, nullptr, st));
   // A4-A8 with the rows of later persons as public zeros, then the rest of the OR tree
   const uint16_t* zcc[3] = {zc[0], zc[1], zc[2]};
   const uint16_t* zmc[3] = {zm[0], zm[1], zm[2]};

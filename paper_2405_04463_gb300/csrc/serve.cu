@@ -2,8 +2,8 @@
 //
 // A request of Q queries occupies Q consecutive query slots of a column pool (R columns per
 // slot, columns q*R + rho as in a stand-alone request). One serving step runs one resident
-// database chunk for every active column: the six share-domain GEMMs (A3, three party streams)
-// and the comparison phase (A4-A8 with the in-block OR) over the column tiles that hold active
+// database chunk for every active column: the six share-domain GEMMs (A3; one launch on the tcgen05
+// paths, three party streams on the int8 ones) and the comparison phase (A4-A8 with the in-block OR) over the column tiles that hold active
 // columns, replayed from a CUDA graph keyed by (chunk, GEMM tile variant); the tile list lives
 // in device memory and is rewritten before each replay, so one graph serves every mix of
 // requests. A request admitted while the loop is at chunk c visits chunks c, c+1, ... and
@@ -46,7 +46,11 @@ struct Variant {
   uint32_t tile_cols;
   int id;  // tcgen05: tile width; int8 paths: ring_gemm_i8_variant index
 };
-const Variant kTcVariants[] = {{"tc256", 256, 256}, {"tc128", 128, 128}};
+// The widths of listed column tiles. 256-column tiles run as two of 128, which the kernel computes at a
+// lower rate than 208-column ones; narrow tiles waste less on a few active columns. The first two can be
+// asked for by number, the others are the autotuner's.
+const Variant kTcVariants[] = {{"tc256", 256, 256}, {"tc128", 128, 128}, {"tc208", 208, 208}, {"tc64", 64, 64}};
+constexpr int kTcFixed = 2;
 const Variant kI8Variants[] = {{"mix128", 128, 0}, {"mma128", 128, 1}, {"mma64", 64, 2}, {"mma32", 32, 3}};
 
 double now_s() {
@@ -142,6 +146,11 @@ uint32_t tile_list(const uint32_t* col0, const uint32_t* ncols, uint32_t n, uint
   return static_cast<uint32_t>(t.size());
 }
 
+// Column tiles of variant v that cover the pool (the last one may reach past it).
+uint32_t tiles_of(const Server& S, int v) {
+  return (S.pool_pad + S.variants[v].tile_cols - 1) / S.variants[v].tile_cols;
+}
+
 int pick_variant(const Server& S, uint32_t active_cols) {
   for (const Bucket& b : S.buckets)
     if (active_cols <= b.cols) return b.variant;
@@ -170,32 +179,45 @@ uint16_t* z_plane(const Server& S, int vec, int party) {
   return S.z + static_cast<size_t>(vec * 3 + party) * S.pool_pad * S.c->cfg.db_chunk_rows;
 }
 
-// A3 of one party and vector over the listed tiles of the pool, for one chunk.
+bool tensor_path(const Server& S) { return S.c->cfg.path == IPC_PATH_TC || S.c->cfg.path == IPC_PATH_TCG; }
+
+// A3 of every party and vector over the listed tiles of the pool, for one chunk (tcgen05 paths):
+// replicated sharing: [own | previous] components, K = 2l; Galois-ring Shamir: own share, K = l.
+// n_pass: the first passes only (one, when the autotuner times a variant).
+int gemm_all(Server& S, int v, const Chunk& ch, uint32_t n_pass, cudaStream_t st) {
+  ipc_ctx* c = S.c;
+  const bool gal = c->cfg.path == IPC_PATH_TCG;
+  auto p16 = [](const uint8_t* p) { return reinterpret_cast<const uint16_t*>(p); };
+  auto p8 = [](const uint8_t* p) { return reinterpret_cast<const int8_t*>(p); };
+  RingGemm g[RING_GEMM_PASSES];
+  for (int vec = 0; vec < 2; ++vec)
+    for (int i = 0; i < 3; ++i) {
+      const int prev = (i + 2) % 3, other = gal ? i : prev;
+      g[3 * vec + i] = RingGemm{{p8(ctx_plane(c, ch, i, vec, 0)), p8(ctx_plane(c, ch, other, vec, 0))},
+                                {p8(ctx_plane(c, ch, i, vec, 1)), p8(ctx_plane(c, ch, other, vec, 1))},
+                                gal ? 1u : 2u,
+                                p16(bq_plane(S, i, vec, 0)),
+                                p16(bq_plane(S, i, vec, 1)),
+                                c->cfg.seeds[i],
+                                c->cfg.seeds[prev],
+                                static_cast<uint32_t>(vec),
+                                z_plane(S, vec, i)};
+    }
+  return ring_gemm_ts(n_pass, g, ch.rows, S.pool_pad, S.pool_pad, c->l, S.tags, c->cfg.db_chunk_rows, ch.row0,
+                      S.variants[v].tile_cols, S.list_dev[v], S.count_dev[v], st);
+}
+
+// A3 of one party and vector over the listed tiles of the pool, for one chunk (int8 paths).
 int gemm(Server& S, int v, const Chunk& ch, int party, int vec, cudaStream_t st) {
   ipc_ctx* c = S.c;
   const int prev = (party + 2) % 3;
-  const Variant& V = S.variants[v];
-  uint16_t* zo = z_plane(S, vec, party);
-  const size_t ldz = c->cfg.db_chunk_rows;
-  if (c->cfg.path == IPC_PATH_TC || c->cfg.path == IPC_PATH_TCG) {
-    // replicated sharing: [own | previous] components, K = 2l; Galois-ring Shamir: own share, K = l
-    const bool gal = c->cfg.path == IPC_PATH_TCG;
-    const int other = gal ? party : prev;
-    auto p16 = [](const uint8_t* p) { return reinterpret_cast<const uint16_t*>(p); };
-    auto p8 = [](const uint8_t* p) { return reinterpret_cast<const int8_t*>(p); };
-    const int8_t* xl[2] = {p8(ctx_plane(c, ch, party, vec, 0)), p8(ctx_plane(c, ch, other, vec, 0))};
-    const int8_t* xh[2] = {p8(ctx_plane(c, ch, party, vec, 1)), p8(ctx_plane(c, ch, other, vec, 1))};
-    return ring_gemm_tc_variant(V.tile_cols, gal ? 1 : 2, xl, xh, ch.rows, p16(bq_plane(S, party, vec, 0)),
-                                p16(bq_plane(S, party, vec, 1)), S.pool_pad, S.pool_pad, c->l, S.tags,
-                                c->cfg.seeds[party], c->cfg.seeds[prev], static_cast<uint32_t>(vec), zo, ldz, ch.row0,
-                                S.list_dev[v], S.count_dev[v], st);
-  }
   auto p8 = [](const uint8_t* p) { return reinterpret_cast<const int8_t*>(p); };
   const int8_t* xl[2] = {p8(ctx_plane(c, ch, party, vec, 0)), p8(ctx_plane(c, ch, prev, vec, 0))};
   const int8_t* xh[2] = {p8(ctx_plane(c, ch, party, vec, 1)), p8(ctx_plane(c, ch, prev, vec, 1))};
-  return ring_gemm_i8_variant(V.id, xl, xh, ch.rows, p8(bq_plane(S, party, vec, 0)), p8(bq_plane(S, party, vec, 1)),
-                              S.pool_pad, S.pool_pad, c->l, S.tags, c->cfg.seeds[party], c->cfg.seeds[prev],
-                              static_cast<uint32_t>(vec), zo, ldz, ch.row0, S.list_dev[v], S.count_dev[v], st);
+  return ring_gemm_i8_variant(S.variants[v].id, xl, xh, ch.rows, p8(bq_plane(S, party, vec, 0)),
+                              p8(bq_plane(S, party, vec, 1)), S.pool_pad, S.pool_pad, c->l, S.tags,
+                              c->cfg.seeds[party], c->cfg.seeds[prev], static_cast<uint32_t>(vec), z_plane(S, vec, party),
+                              c->cfg.db_chunk_rows, ch.row0, S.list_dev[v], S.count_dev[v], st);
 }
 
 int compare(Server& S, int v, const Chunk& ch, cudaStream_t st) {
@@ -206,8 +228,8 @@ int compare(Server& S, int v, const Chunk& ch, cudaStream_t st) {
                               S.count_dev[v], S.variants[v].tile_cols, st, nullptr, S.c->cfg.plain_mask != 0);
 }
 
-// The graph of one step: fork the party streams off the control stream, two GEMMs per party,
-// join, then the comparison phase on the control stream.
+// The graph of one step: the GEMMs (int8 paths: fork the party streams off the control stream, two
+// GEMMs per party, join), then the comparison phase on the control stream.
 int step_graph(Server& S, uint32_t chunk, int v, cudaGraphExec_t* out) {
   auto it = S.graphs.find({chunk, v});
   if (it != S.graphs.end()) {
@@ -219,8 +241,13 @@ int step_graph(Server& S, uint32_t chunk, int v, cudaGraphExec_t* out) {
   cudaGraph_t g = nullptr;
   SRV_TRY(cudaStreamBeginCapture(c->sc, cudaStreamCaptureModeThreadLocal));
   int rc = IPC_OK;
-  cudaError_t e = cudaEventRecord(S.ev_fork, c->sc);
-  for (int i = 0; i < 3 && e == cudaSuccess && rc == IPC_OK; ++i) {
+  const bool joint = tensor_path(S);
+  cudaError_t e = cudaSuccess;
+  if (joint)
+    rc = gemm_all(S, v, ch, RING_GEMM_PASSES, c->sc);
+  else
+    e = cudaEventRecord(S.ev_fork, c->sc);
+  for (int i = 0; !joint && i < 3 && e == cudaSuccess && rc == IPC_OK; ++i) {
     e = cudaStreamWaitEvent(c->sp[i], S.ev_fork, 0);
     for (int vec = 0; vec < 2 && e == cudaSuccess && rc == IPC_OK; ++vec) rc = gemm(S, v, ch, i, vec, c->sp[i]);
     if (e == cudaSuccess && rc == IPC_OK) e = cudaEventRecord(S.ev_join[i], c->sp[i]);
@@ -333,7 +360,7 @@ int run_step(Server& S, uint64_t step, const std::vector<SReq*>& admitted) {
   }
   const int v = pick_variant(S, active_cols);
   const uint32_t tw = S.variants[v].tile_cols;
-  std::vector<uint32_t> tiles(S.pool_pad / tw);
+  std::vector<uint32_t> tiles(tiles_of(S, v));
   tiles.resize(tile_list(c0.data(), nc.data(), static_cast<uint32_t>(c0.size()), tw, tiles.data(),
                          static_cast<uint32_t>(tiles.size())));
   SRV_RC(upload_list(S, v, tiles, step));
@@ -406,7 +433,7 @@ void worker_main(Server* Sp) {
 
 // ---------------------------------------------------------------------------------------------
 // Autotuner: per bucket of active columns, the GEMM variant with the shortest launch over the
-// first resident chunk, one party and vector, the listed tiles covering that many columns.
+// first resident chunk, the listed tiles covering that many columns.
 // The table is cached as JSON keyed by device, geometry, chunk rows, path and pool width.
 // ---------------------------------------------------------------------------------------------
 
@@ -415,7 +442,7 @@ std::string tune_key(const Server& S) {
   cudaGetDeviceProperties(&prop, S.c->cfg.device);
   std::ostringstream k;
   k << prop.name << "|sm" << prop.multiProcessorCount << "|l" << S.c->l << "|rows" << S.c->cfg.db_chunk_rows << "|path"
-    << S.c->cfg.path << "|pool" << S.pool_pad;
+    << S.c->cfg.path << "|pool" << S.pool_pad << "|v" << S.n_variants;
   return k.str();
 }
 
@@ -460,26 +487,32 @@ int autotune(Server& S) {
   js << "{\"key\": \"" << key << "\", \"buckets\": [";
   std::vector<Bucket> b;
   bool first = true;
-  for (uint32_t cols = kPoolAlign; ; cols *= 2) {
+  // tcgen05: the narrow tiles are candidates while one of them, or two, cover the active columns (they
+  // compute at a lower rate), the wide ones above that
+  const bool joint = tensor_path(S);
+  for (uint32_t cols = joint ? 64 : kPoolAlign; ; cols *= 2) {
     const uint32_t w = std::min(cols, S.pool_pad);
     float best = 1e30f;
     int best_v = 0;
     std::ostringstream ms;
     for (int v = 0; v < S.n_variants; ++v) {
       const uint32_t tw = S.variants[v].tile_cols;
+      if (joint && (w <= 128) != (tw <= 128)) continue;
       std::vector<uint32_t> tiles((w + tw - 1) / tw);
       for (uint32_t k = 0; k < tiles.size(); ++k) tiles[k] = k;
       SRV_RC(upload_list(S, v, tiles, 0));
       SRV_TRY(cudaStreamSynchronize(c->sc));
-      SRV_RC(gemm(S, v, ch, 0, 0, c->sc));  // warm-up (also sets the kernel attributes before any capture)
+      // one party and vector, warmed up (which also sets the kernel attributes before any capture)
+      auto once = [&] { return joint ? gemm_all(S, v, ch, 1, c->sc) : gemm(S, v, ch, 0, 0, c->sc); };
+      SRV_RC(once());
       SRV_TRY(cudaEventRecord(e0, c->sc));
-      for (int rep = 0; rep < 2; ++rep) SRV_RC(gemm(S, v, ch, 0, 0, c->sc));
+      for (int rep = 0; rep < 2; ++rep) SRV_RC(once());
       SRV_TRY(cudaEventRecord(e1, c->sc));
       SRV_TRY(cudaEventSynchronize(e1));
       float t = 0;
       SRV_TRY(cudaEventElapsedTime(&t, e0, e1));
       t /= 2;
-      ms << (v ? ", " : "") << "\"" << S.variants[v].name << "\": " << t;
+      ms << (ms.tellp() > 0 ? ", " : "") << "\"" << S.variants[v].name << "\": " << t;
       if (t < best) {
         best = t;
         best_v = v;
@@ -602,8 +635,8 @@ extern "C" int ipc_serve_start(ipc_ctx* c, const ipc_serve_config* cfg) {
   S.cfg = *cfg;
   const bool tc = c->cfg.path == IPC_PATH_TC || c->cfg.path == IPC_PATH_TCG;
   S.variants = tc ? kTcVariants : kI8Variants;
-  S.n_variants = tc ? 2 : 4;
-  if (cfg->variant != IPC_SERVE_AUTOTUNE && (cfg->variant < 0 || cfg->variant >= S.n_variants)) {
+  S.n_variants = 4;
+  if (cfg->variant != IPC_SERVE_AUTOTUNE && (cfg->variant < 0 || cfg->variant >= (tc ? kTcFixed : S.n_variants))) {
     delete Sp;
     return ctx_fail(c, IPC_EINVAL, "ipc_serve_start: unknown variant");
   }
@@ -643,7 +676,7 @@ extern "C" int ipc_serve_start(ipc_ctx* c, const ipc_serve_config* cfg) {
   for (int v = 0; v < S.n_variants && ok; ++v) {
     uint32_t* ld = nullptr;
     uint32_t* cd = nullptr;
-    ok = cudaMalloc(&ld, (S.pool_pad / S.variants[v].tile_cols) * sizeof(uint32_t)) == cudaSuccess &&
+    ok = cudaMalloc(&ld, tiles_of(S, v) * sizeof(uint32_t)) == cudaSuccess &&
          cudaMalloc(&cd, sizeof(uint32_t)) == cudaSuccess;
     S.list_dev.push_back(ld);
     S.count_dev.push_back(cd);
@@ -671,7 +704,7 @@ extern "C" int ipc_serve_start(ipc_ctx* c, const ipc_serve_config* cfg) {
       rc = autotune(S);
     } else {
       // warm-up launch of the chosen variant (kernel attributes are set outside any capture)
-      rc = gemm(S, cfg->variant, c->chunks[0], 0, 0, c->sc);
+      rc = tc ? gemm_all(S, cfg->variant, c->chunks[0], 1, c->sc) : gemm(S, cfg->variant, c->chunks[0], 0, 0, c->sc);
     }
   }
   if (rc == IPC_OK) {

@@ -89,6 +89,13 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// True for one lane of a converged warp, the same one each time.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r != 0;
+}
+
 // 32 consecutive TMEM columns of this thread's lane.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -136,6 +143,8 @@ __device__ __forceinline__ uint32_t add16x2(uint32_t a, uint32_t b) {
   asm("add.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
 }
+
+__device__ __forceinline__ uint32_t sub16x2(uint32_t a, uint32_t b) { return add16x2(a, add16x2(~b, 0x00010001u)); }
 
 // Low 16 bits of x (lane 0) and of y (lane 1): the L contributions of two columns.
 __device__ __forceinline__ uint32_t pack_lo16(uint32_t x, uint32_t y) {
@@ -238,10 +247,11 @@ inline PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// fp16 tensor [rows][cols] (row stride cols * 2 bytes) as a TMA tensor map: box 32 elements
-// (one 64-byte swizzled row) x box_rows, 64-byte swizzle, zero fill outside the tensor (query
-// rows past n_pad).
-inline int make_map_f16(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_rows) {
+// fp16 tensor [rows][cols] (row stride cols * 2 bytes) as a TMA tensor map: box BOX elements (one
+// swizzled row of 64 or 128 bytes) x box_rows, zero fill outside the tensor (query rows past n_pad).
+template <uint32_t BOX>
+int make_map_f16_box(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_rows) {
+  static_assert(BOX == 32 || BOX == 64, "box of 64 or 128 bytes");
   auto fn = encode_fn();
   if (!fn) {
     set_error("cuTensorMapEncodeTiled is not available from the driver");
@@ -249,16 +259,22 @@ inline int make_map_f16(CUtensorMap* map, const void* base, uint64_t cols, uint6
   }
   cuuint64_t dims[2] = {cols, rows};
   cuuint64_t strides[1] = {cols * 2};
-  cuuint32_t box[2] = {32, box_rows};
+  cuuint32_t box[2] = {BOX, box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, BOX == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_error("cuTensorMapEncodeTiled (fp16) failed with CUresult " + std::to_string(static_cast<int>(r)));
     return IPC_ECUDA;
   }
   return IPC_OK;
+}
+inline int make_map_f16(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_rows) {
+  return make_map_f16_box<32>(map, base, cols, rows, box_rows);
+}
+inline int make_map_f16k64(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_rows) {
+  return make_map_f16_box<64>(map, base, cols, rows, box_rows);
 }
 
 // int8 limb plane [rows][cols] (row stride cols bytes, a multiple of 16) as a TMA tensor map:
@@ -279,6 +295,31 @@ inline int make_map_i8(CUtensorMap* map, const void* base, uint64_t cols, uint64
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_error("cuTensorMapEncodeTiled (int8) failed with CUresult " + std::to_string(static_cast<int>(r)));
+    return IPC_ECUDA;
+  }
+  return IPC_OK;
+}
+
+// int8 limb plane [rows][cols] as a TMA tensor map of raw tiles: box box_cols (64 or 128) bytes x
+// box_rows, rows swizzled at their width (16-byte chunk c of row r at position c ^ ((r >> 1) & 3) or
+// c ^ (r & 7)), zero fill past the last row.
+inline int make_map_raw(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_cols,
+                        uint32_t box_rows) {
+  auto fn = encode_fn();
+  if (!fn) {
+    set_error("cuTensorMapEncodeTiled is not available from the driver");
+    return IPC_ECUDA;
+  }
+  cuuint64_t dims[2] = {cols, rows};
+  cuuint64_t strides[1] = {cols};
+  cuuint32_t box[2] = {box_cols, box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    set_error("cuTensorMapEncodeTiled (raw int8) failed with CUresult " + std::to_string(static_cast<int>(r)));
     return IPC_ECUDA;
   }
   return IPC_OK;
