@@ -16,22 +16,37 @@ namespace ipc {
 // XORed with the other counter words and the round key; the key advances by
 // the Weyl increments 0x9E3779B9 / 0xBB67AE85 between rounds.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint64_t seed) {
-  uint32_t k0 = static_cast<uint32_t>(seed), k1 = static_cast<uint32_t>(seed >> 32);
+// The round keys of a seed. Kernels that draw many blocks take them as launch parameters: a round is
+// then two wide products and two three-input xors with the key as a constant-bank operand, four
+// instructions where advancing the key costs two more.
+struct PhiloxKey {
+  uint32_t k[20];
+};
+
+__host__ __device__ inline PhiloxKey philox_key(uint64_t seed) {
+  PhiloxKey key;
+  for (int r = 0; r < 10; ++r) {
+    key.k[2 * r] = static_cast<uint32_t>(seed) + static_cast<uint32_t>(r) * 0x9E3779B9u;
+    key.k[2 * r + 1] = static_cast<uint32_t>(seed >> 32) + static_cast<uint32_t>(r) * 0xBB67AE85u;
+  }
+  return key;
+}
+
+__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const PhiloxKey& key) {
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
     const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
     const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
-    const uint32_t n0 = hi1 ^ c1 ^ k0;
-    const uint32_t n2 = hi0 ^ c3 ^ k1;
-    c0 = n0;
+    c0 = hi1 ^ c1 ^ key.k[2 * r];
+    c2 = hi0 ^ c3 ^ key.k[2 * r + 1];
     c1 = lo1;
-    c2 = n2;
     c3 = lo0;
-    k0 += 0x9E3779B9u;
-    k1 += 0xBB67AE85u;
   }
   return make_uint4(c0, c1, c2, c3);
+}
+
+__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint64_t seed) {
+  return philox(c0, c1, c2, c3, philox_key(seed));
 }
 
 __device__ __forceinline__ uint32_t word_of(const uint4& w, uint32_t i) {

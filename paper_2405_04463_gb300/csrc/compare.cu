@@ -17,15 +17,16 @@ namespace {
 using namespace cmp;
 
 constexpr int CT = 64;  // threads per CTA
+constexpr uint64_t PLAIN_THREADS = 300000;  // about four times what the chip holds at once
 // One thread per part of each (column, OR block) unit, the parts of a unit in consecutive lanes,
 // joined by warp shuffles; the modes are those of part_root.
 template <int MODE>
-__global__ void __launch_bounds__(CT) compare_kernel(const CmpParams P) {
+__global__ void __launch_bounds__(CT) compare_kernel(const __grid_constant__ CmpParams P, const __grid_constant__ Seeds sd) {
   extern __shared__ uint32_t sm[];  // [S_WORDS][CT]
   const uint32_t tid = threadIdx.x;
   const uint64_t gtid = blockIdx.x * static_cast<uint64_t>(CT) + tid;
   // all threads of a unit leave together, so the group stays complete for the final shuffles
-  const uint32_t ks = P.p < LOG2_SPLIT ? P.p : LOG2_SPLIT;
+  const uint32_t ks = P.ks;
   const uint64_t unit = gtid >> ks;
   const uint32_t part = static_cast<uint32_t>(gtid & ((1u << ks) - 1u));
   if (unit >= static_cast<uint64_t>(P.n_cols) * P.n_blocks) return;
@@ -40,14 +41,14 @@ __global__ void __launch_bounds__(CT) compare_kernel(const CmpParams P) {
   }
   B3 root;
   uint32_t nwords;
-  part_root<MODE, CT>(P, n, blk, part, ks, sm, tid, root, nwords);
+  part_root<MODE, CT>(P, sd, n, blk, part, ks, sm, tid, root, nwords);
   const uint32_t req = P.col_tags[2 * n], tag = P.col_tags[2 * n + 1];
   const uint32_t sub_p = P.p - ks;
   const uint64_t bword0 = (P.row0 + (static_cast<uint64_t>(blk) << (5 + P.p))) >> 5;  // the block's first word
   // ---- join the parts: at step s, part t (t a multiple of 2^s) is the left child and part
   // t + 2^(s-1) the right child of the level sub_p + s node; a part without words is carried
   // (words fill the parts from the first, so a right child with words has a left one). ----
-  const uint32_t group_mask = ((1u << (1u << ks)) - 1u) << (tid & (32u - (1u << ks)));
+  const uint32_t group_mask = ks == 5 ? 0xFFFFFFFFu : ((1u << (1u << ks)) - 1u) << (tid & (32u - (1u << ks)));
   uint32_t has = nwords > 0 ? 1u : 0u;
   for (uint32_t s = 1; s <= ks; ++s) {
     const uint32_t d = 1u << (s - 1);
@@ -58,7 +59,7 @@ __global__ void __launch_bounds__(CT) compare_kernel(const CmpParams P) {
     const uint32_t right_has = __shfl_xor_sync(group_mask, has, d);
     if ((part & ((2u << (s - 1)) - 1u)) == 0 && right_has) {
       const uint32_t lvl = sub_p + s;
-      root = bor(P.seeds, root, right, static_cast<uint32_t>((bword0 >> lvl) + (part >> s)), tag, req,
+      root = bor(sd, root, right, static_cast<uint32_t>((bword0 >> lvl) + (part >> s)), tag, req,
                  (IPC_D_OR << 24) | (1u << 16) | lvl);
     }
     has |= right_has;
@@ -70,34 +71,6 @@ __global__ void __launch_bounds__(CT) compare_kernel(const CmpParams P) {
   P.roots[at] = root.c0;
   P.roots[plane + at] = root.c1;
   P.roots[2 * plane + at] = root.c2;
-}
-
-// Rows stage of the OR tree above the block roots: per column, pairwise levels p+1, p+2, ...
-__global__ void or_rows_kernel(uint32_t* roots, uint64_t ld_roots, uint64_t plane, uint32_t n_cols, uint32_t n_blocks,
-                               uint32_t p, const uint32_t* col_tags, Seeds sd) {
-  const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= n_cols) return;
-  const uint32_t req = col_tags[2 * n], tag = col_tags[2 * n + 1];
-  uint32_t* r0 = roots + static_cast<uint64_t>(n) * ld_roots;
-  uint32_t cnt = n_blocks, level = p + 1;
-  while (cnt > 1) {
-    const uint32_t half = cnt / 2;
-    for (uint32_t j = 0; j < half; ++j) {
-      const B3 a = {r0[2 * j], r0[plane + 2 * j], r0[2 * plane + 2 * j]};
-      const B3 b = {r0[2 * j + 1], r0[plane + 2 * j + 1], r0[2 * plane + 2 * j + 1]};
-      const B3 c = bor(sd, a, b, j, tag, req, (IPC_D_OR << 24) | (1u << 16) | level);
-      r0[j] = c.c0;
-      r0[plane + j] = c.c1;
-      r0[2 * plane + j] = c.c2;
-    }
-    if (cnt & 1u) {
-      r0[half] = r0[cnt - 1];
-      r0[plane + half] = r0[plane + cnt - 1];
-      r0[2 * plane + half] = r0[2 * plane + cnt - 1];
-    }
-    cnt = half + (cnt & 1u);
-    ++level;
-  }
 }
 
 // Block roots from the part roots of the fused GEMM + comparison kernel: per (column, 1,024-row
@@ -140,26 +113,68 @@ __global__ void or_join_parts_kernel(const uint32_t* parts, uint64_t ld_parts, u
   roots[2 * roots_plane + at] = r[0].c2;
 }
 
-// Rotation stage and lane fold, per query.
-__global__ void or_queries_kernel(const uint32_t* roots, uint64_t ld_roots, uint64_t plane, uint32_t Q, uint32_t R,
-                                  const uint32_t* col_tags, Seeds sd, uint8_t* bit_shares) {
-  const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= Q) return;
+// The OR tree above the block roots, one CTA per query: a warp per rotation takes the column's rows
+// stage (pairwise levels p + 1, p + 2, ... in place: a batch of 32 pairs is read before any of its nodes
+// is written, and a node lies before every pair still to be read), then the first warp the rotation
+// stage by shuffles and the fold of the 32 lanes. Bound by the chain of dependent gates (three Philox
+// blocks each): a level costs one of them per 32 pairs where one thread per column walked every pair.
+// 64 blocks x 992 columns: 13 us against 68 us as two kernels of one thread per column and query.
+__global__ void __launch_bounds__(32 * 31) or_tree_kernel(uint32_t* roots, uint64_t ld_roots, uint64_t plane, uint32_t n_blocks,
+                                                          uint32_t p, uint32_t Q, uint32_t R, const uint32_t* col_tags,
+                                                          const __grid_constant__ Seeds sd, uint8_t* bit_shares) {
+  __shared__ B3 cols[32];
+  const uint32_t q = blockIdx.x, rho = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+  {
+    const uint32_t n = q * R + rho, req = col_tags[2 * n], tag = col_tags[2 * n + 1];
+    uint32_t* r0 = roots + static_cast<uint64_t>(n) * ld_roots;
+    uint32_t cnt = n_blocks, level = p + 1;
+    while (cnt > 1) {
+      const uint32_t half = cnt / 2;
+      for (uint32_t j0 = 0; j0 < half; j0 += 32) {
+        const uint32_t j = j0 + lane;
+        B3 a{}, b{};
+        if (j < half) {
+          a = {r0[2 * j], r0[plane + 2 * j], r0[2 * plane + 2 * j]};
+          b = {r0[2 * j + 1], r0[plane + 2 * j + 1], r0[2 * plane + 2 * j + 1]};
+        }
+        __syncwarp();
+        if (j < half) {
+          const B3 c = bor(sd, a, b, j, tag, req, (IPC_D_OR << 24) | (1u << 16) | level);
+          r0[j] = c.c0;
+          r0[plane + j] = c.c1;
+          r0[2 * plane + j] = c.c2;
+        }
+        __syncwarp();
+      }
+      if ((cnt & 1u) && lane == 0) {
+        r0[half] = r0[cnt - 1];
+        r0[plane + half] = r0[plane + cnt - 1];
+        r0[2 * plane + half] = r0[2 * plane + cnt - 1];
+      }
+      __syncwarp();
+      cnt = half + (cnt & 1u);
+      ++level;
+    }
+    if (lane == 0) cols[rho] = {r0[0], r0[plane], r0[2 * plane]};
+  }
+  __syncthreads();
+  if (rho != 0) return;
   const uint32_t req = col_tags[2 * (q * R)], tag = col_tags[2 * (q * R) + 1] & ~31u;
-  B3 w[32];
-  for (uint32_t rho = 0; rho < R; ++rho) {
-    const uint64_t at = static_cast<uint64_t>(q * R + rho) * ld_roots;
-    w[rho] = {roots[at], roots[plane + at], roots[2 * plane + at]};
-  }
-  uint32_t cnt = R, level = 1;
-  while (cnt > 1) {
+  B3 w = lane < R ? cols[lane] : B3{0u, 0u, 0u};
+  auto from = [&](uint32_t src) {
+    return B3{__shfl_sync(0xFFFFFFFFu, w.c0, src), __shfl_sync(0xFFFFFFFFu, w.c1, src), __shfl_sync(0xFFFFFFFFu, w.c2, src)};
+  };
+  for (uint32_t cnt = R, level = 1; cnt > 1; ++level) {
     const uint32_t half = cnt / 2;
-    for (uint32_t j = 0; j < half; ++j) w[j] = bor(sd, w[2 * j], w[2 * j + 1], j, tag, req, (IPC_D_OR << 24) | (2u << 16) | level);
-    if (cnt & 1u) w[half] = w[cnt - 1];
+    const B3 a = from((2 * lane) & 31u), b = from((2 * lane + 1) & 31u), last = from(cnt - 1);
+    if (lane < half)
+      w = bor(sd, a, b, lane, tag, req, (IPC_D_OR << 24) | (2u << 16) | level);
+    else if (lane == half)
+      w = last;  // an odd last node moves up; with an even count nothing reads it
     cnt = half + (cnt & 1u);
-    ++level;
   }
-  B3 x = w[0];
+  if (lane != 0) return;
+  B3 x = w;
   for (uint32_t L = 1; L <= 5; ++L) {
     const uint32_t h = 32u >> L;
     const uint32_t m = (1u << h) - 1u;
@@ -173,13 +188,22 @@ __global__ void or_queries_kernel(const uint32_t* roots, uint64_t ld_roots, uint
   bit_shares[2 * Q + q] = x.c2 & 1u;
 }
 
-int launch_compare(CmpParams& P, int mode, cudaStream_t st) {
+int launch_compare(CmpParams& P, const uint64_t seeds[3], int mode, cudaStream_t st) {
   if (P.p > 5) {  // a part's OR stack holds levels 0..5 - LOG2_SPLIT
     set_error("compare: log2_block_words must be <= 5");
     return IPC_EINVAL;
   }
   P.n_blocks = static_cast<uint32_t>((P.n_rows + (32ull << P.p) - 1) >> (5 + P.p));
-  const uint64_t threads = (static_cast<uint64_t>(P.n_cols) * P.n_blocks) << (P.p < LOG2_SPLIT ? P.p : LOG2_SPLIT);
+  // Threads per unit: one per 32-row word. Eight threads of four words each leave small launches short of
+  // warps (1,000 rows x 4 columns: 62 us with 8, 23 us with 32; 65,536 x 31: 64 and 43 us) and read a
+  // column with gaps; at 65,536 x 992 the lift takes 994 us with 8 (seeds advanced in the kernel) and
+  // 946 us with 32. Protocol 1's short comparison is bound by its loads' and joins' overhead once warps
+  // abound: 271 us with 8 threads against 297 us with 32, so it takes 32 only below that.
+  const uint64_t units = static_cast<uint64_t>(P.n_cols) * P.n_blocks;
+  P.ks = mode == MODE_PLAIN ? (P.p < LOG2_SPLIT ? P.p : LOG2_SPLIT) : P.p;
+  while (P.ks < P.p && (units << P.ks) < PLAIN_THREADS) ++P.ks;
+  const uint64_t threads = units << P.ks;
+  const Seeds sd = make_seeds(seeds);
   const size_t smem = sizeof(uint32_t) * S_WORDS * CT;
   static tc::PerDevice attr;  // a kernel attribute belongs to one device's context
   IPC_CUDA_TRY(attr.run([smem] {
@@ -195,20 +219,18 @@ int launch_compare(CmpParams& P, int mode, cudaStream_t st) {
   }));
   const unsigned grid = static_cast<unsigned>((threads + CT - 1) / CT);
   if (mode == MODE_PLAIN)
-    compare_kernel<MODE_PLAIN><<<grid, CT, smem, st>>>(P);
+    compare_kernel<MODE_PLAIN><<<grid, CT, smem, st>>>(P, sd);
   else if (mode == MODE_LIFTFREE)
-    compare_kernel<MODE_LIFTFREE><<<grid, CT, smem, st>>>(P);
+    compare_kernel<MODE_LIFTFREE><<<grid, CT, smem, st>>>(P, sd);
   else
-    compare_kernel<MODE_LIFT><<<grid, CT, smem, st>>>(P);
+    compare_kernel<MODE_LIFT><<<grid, CT, smem, st>>>(P, sd);
   IPC_CUDA_TRY(cudaGetLastError());
   return IPC_OK;
 }
 
 CmpParams base_params(size_t ldz, uint32_t n_cols, size_t n_rows, uint64_t row0, const uint32_t* col_tags,
-                      const uint64_t seeds[3], uint32_t thr_a, uint32_t p, uint32_t* roots, size_t ld_roots,
-                      uint8_t* msb_out, size_t ld_msb) {
+                      uint32_t thr_a, uint32_t p, uint32_t* roots, size_t ld_roots, uint8_t* msb_out, size_t ld_msb) {
   CmpParams P{};
-  for (int j = 0; j < 3; ++j) P.seeds.s[j] = seeds[j];
   P.ldz = ldz;
   P.n_cols = n_cols;
   P.n_rows = n_rows;
@@ -230,7 +252,7 @@ int compare_launch_tiles(const uint16_t* const z_code[3], const uint16_t* const 
                          const uint64_t seeds[3], uint32_t thr_a, uint32_t p, uint32_t* roots, size_t ld_roots,
                          uint8_t* msb_out, size_t ld_msb, const uint32_t* col_tiles, const uint32_t* n_col_list,
                          uint32_t tile_cols, cudaStream_t st, const uint32_t* col_rows, bool plain) {
-  CmpParams P = base_params(ldz, n_cols, n_rows, row0, col_tags, seeds, thr_a, p, roots, ld_roots, msb_out, ld_msb);
+  CmpParams P = base_params(ldz, n_cols, n_rows, row0, col_tags, thr_a, p, roots, ld_roots, msb_out, ld_msb);
   for (int j = 0; j < 3; ++j) {
     P.zc[j] = z_code[j];
     P.zm[j] = z_mask[j];
@@ -239,7 +261,7 @@ int compare_launch_tiles(const uint16_t* const z_code[3], const uint16_t* const 
   P.n_col_list = n_col_list;
   P.tile_cols = tile_cols;
   P.col_rows = col_rows;
-  return launch_compare(P, plain ? MODE_PLAIN : MODE_LIFT, st);
+  return launch_compare(P, seeds, plain ? MODE_PLAIN : MODE_LIFT, st);
 }
 
 // ConstLift (zc16 set, zc32 null) or NoLift (zc32 set): ml32 the Z_2^32 components of ml.
@@ -248,14 +270,14 @@ int compare_launch_liftfree(const uint16_t* const zc16[3], const uint32_t* const
                             const uint32_t* col_tags, const uint64_t seeds[3], uint32_t thr_a, uint32_t thr_b,
                             uint32_t p, uint32_t* roots, size_t ld_roots, uint8_t* msb_out, size_t ld_msb,
                             cudaStream_t st) {
-  CmpParams P = base_params(ldz, n_cols, n_rows, row0, col_tags, seeds, thr_a, p, roots, ld_roots, msb_out, ld_msb);
+  CmpParams P = base_params(ldz, n_cols, n_rows, row0, col_tags, thr_a, p, roots, ld_roots, msb_out, ld_msb);
   for (int j = 0; j < 3; ++j) {
     P.zc[j] = zc16 ? zc16[j] : nullptr;
     P.zc32[j] = zc32 ? zc32[j] : nullptr;
     P.zm32[j] = ml32[j];
   }
   P.thr_b = zc32 ? (thr_b == 0 ? 65536u : thr_b) : 65536u;
-  return launch_compare(P, MODE_LIFTFREE, st);
+  return launch_compare(P, seeds, MODE_LIFTFREE, st);
 }
 
 int compare_launch(const uint16_t* const z_code[3], const uint16_t* const z_mask[3], size_t ldz, uint32_t n_cols,
@@ -270,8 +292,7 @@ int compare_launch(const uint16_t* const z_code[3], const uint16_t* const z_mask
 int or_join_parts_launch(const uint32_t* parts, size_t ld_parts, uint32_t n_cols, size_t n_rows, uint64_t row0,
                          const uint32_t* col_tags, const uint64_t seeds[3], uint32_t* roots, size_t ld_roots,
                          cudaStream_t st) {
-  Seeds sd;
-  for (int j = 0; j < 3; ++j) sd.s[j] = seeds[j];
+  const Seeds sd = make_seeds(seeds);
   const uint64_t n_rt = (n_rows + 127) / 128;
   const uint32_t n_blocks = static_cast<uint32_t>((n_rows + 1023) / 1024);
   const uint64_t units = static_cast<uint64_t>(n_cols) * n_blocks;
@@ -288,12 +309,8 @@ int or_join_parts_launch(const uint32_t* parts, size_t ld_parts, uint32_t n_cols
 int or_finalize_strided(uint32_t* roots, size_t ld_roots, size_t plane, uint32_t n_blocks, uint32_t p, uint32_t Q,
                         uint32_t R, const uint32_t* col_tags, const uint64_t seeds[3], uint8_t* bit_shares,
                         cudaStream_t st) {
-  Seeds sd;
-  for (int j = 0; j < 3; ++j) sd.s[j] = seeds[j];
-  const uint32_t n_cols = Q * R;
-  or_rows_kernel<<<(n_cols + 127) / 128, 128, 0, st>>>(roots, ld_roots, plane, n_cols, n_blocks, p, col_tags, sd);
-  IPC_CUDA_TRY(cudaGetLastError());
-  or_queries_kernel<<<(Q + 63) / 64, 64, 0, st>>>(roots, ld_roots, plane, Q, R, col_tags, sd, bit_shares);
+  const Seeds sd = make_seeds(seeds);
+  or_tree_kernel<<<Q, 32 * R, 0, st>>>(roots, ld_roots, plane, n_blocks, p, Q, R, col_tags, sd, bit_shares);
   IPC_CUDA_TRY(cudaGetLastError());
   return IPC_OK;
 }
@@ -307,9 +324,9 @@ __global__ void or_combine_kernel(const uint8_t* b0, const uint8_t* b1, const ui
   if (p >= P) return;
   auto load = [&](const uint8_t* b) { return B3{b[p] & 1u, b[P + p] & 1u, b[2 * P + p] & 1u}; };
   auto gate = [&](const B3& x, const B3& y, uint32_t t) {
-    const uint32_t F0 = philox(p, 0u, req, (IPC_D_COMB << 24) | t, sd.s[0]).x & 1u;
-    const uint32_t F1 = philox(p, 0u, req, (IPC_D_COMB << 24) | t, sd.s[1]).x & 1u;
-    const uint32_t F2 = philox(p, 0u, req, (IPC_D_COMB << 24) | t, sd.s[2]).x & 1u;
+    const uint32_t F0 = philox(p, 0u, req, (IPC_D_COMB << 24) | t, sd.k[0]).x & 1u;
+    const uint32_t F1 = philox(p, 0u, req, (IPC_D_COMB << 24) | t, sd.k[1]).x & 1u;
+    const uint32_t F2 = philox(p, 0u, req, (IPC_D_COMB << 24) | t, sd.k[2]).x & 1u;
     return bx(bx(x, y), band(x, y, F0, F1, F2));
   };
   const B3 left = gate(load(b0), load(b1), 0), right = gate(load(b2), load(b3), 1);
@@ -321,8 +338,7 @@ __global__ void or_combine_kernel(const uint8_t* b0, const uint8_t* b1, const ui
 
 int or_combine_launch(const uint8_t* const bits[4], uint32_t P, uint32_t req, const uint64_t seeds[3], uint8_t* out,
                       cudaStream_t st) {
-  Seeds sd;
-  for (int j = 0; j < 3; ++j) sd.s[j] = seeds[j];
+  const Seeds sd = make_seeds(seeds);
   or_combine_kernel<<<(P + 127) / 128, 128, 0, st>>>(bits[0], bits[1], bits[2], bits[3], P, req, sd, out);
   IPC_CUDA_TRY(cudaGetLastError());
   return IPC_OK;

@@ -30,8 +30,12 @@ __device__ __forceinline__ B3 band(const B3& x, const B3& y, uint32_t F0, uint32
 }
 
 struct Seeds {
-  uint64_t s[3];
+  PhiloxKey k[3];  // of the seeds shared by parties j and j + 1
 };
+
+__host__ __device__ inline Seeds make_seeds(const uint64_t seeds[3]) {
+  return {{philox_key(seeds[0]), philox_key(seeds[1]), philox_key(seeds[2])}};
+}
 
 // Zero-share words of the AND gates of one 32-row word: gate G uses word (G & 3) of
 // Philox(seed_j, (g >> 5, tag, req, D_AND << 24 | G >> 2)).
@@ -40,7 +44,7 @@ struct GateRng {
   uint4 w[3];
   __device__ __forceinline__ void refresh(const Seeds& sd, uint32_t quad) {
 #pragma unroll
-    for (int j = 0; j < 3; ++j) w[j] = philox(c0, tag, req, (IPC_D_AND << 24) | quad, sd.s[j]);
+    for (int j = 0; j < 3; ++j) w[j] = philox(c0, tag, req, (IPC_D_AND << 24) | quad, sd.k[j]);
   }
   __device__ __forceinline__ void get(const Seeds& sd, uint32_t gate, bool first, uint32_t& F0, uint32_t& F1,
                                       uint32_t& F2) {
@@ -113,9 +117,9 @@ struct CmpParams {
   uint64_t n_rows;
   uint64_t row0;
   const uint32_t* col_tags;
-  Seeds seeds;
   uint32_t thr_a;
-  uint32_t p;  // log2 words per block
+  uint32_t p;   // log2 words per block
+  uint32_t ks;  // log2 threads per block (at most p)
   uint32_t n_blocks;
   uint32_t* roots;
   uint64_t ld_roots;
@@ -134,11 +138,11 @@ struct CmpParams {
 
 constexpr int MODE_LIFT = 0, MODE_PLAIN = 1, MODE_LIFTFREE = 2;
 
-// 2^ks threads share one (column, OR block), ks = min(LOG2_SPLIT, p): thread t takes the t-th
-// part of the block's words (a level sub_p = p - ks subtree) and the group joins the parts
+// 2^ks threads share one (column, OR block), ks chosen at launch (at least LOG2_SPLIT where p is):
+// thread t takes the t-th part of the block's words (a level sub_p = p - ks subtree) and the group joins the parts
 // pairwise with the block's upper ks levels of OR gates. Gate indices are global node indices
 // at each level, so the tree and every share are the same as one thread walking the whole
-// block. With 1,024-row blocks each thread takes 4 words.
+// block. With 1,024-row blocks and ks = 3 each thread takes 4 words.
 constexpr uint32_t LOG2_SPLIT = 3;
 
 // Shared memory per thread (index [slot][threadIdx.x], conflict-free): X, 3 x 32 words (per
@@ -148,9 +152,9 @@ constexpr int S_X = 0, S_STK = 96, S_WORDS = S_STK + 3 * (6 - static_cast<int>(L
 
 __device__ __forceinline__ B3 bor(const Seeds& sd, const B3& a, const B3& b, uint32_t j, uint32_t tag, uint32_t req,
                                   uint32_t c3) {
-  const uint32_t F0 = philox(j, tag, req, c3, sd.s[0]).x;
-  const uint32_t F1 = philox(j, tag, req, c3, sd.s[1]).x;
-  const uint32_t F2 = philox(j, tag, req, c3, sd.s[2]).x;
+  const uint32_t F0 = philox(j, tag, req, c3, sd.k[0]).x;
+  const uint32_t F1 = philox(j, tag, req, c3, sd.k[1]).x;
+  const uint32_t F2 = philox(j, tag, req, c3, sd.k[2]).x;
   return bx(bx(a, b), band(a, b, F0, F1, F2));
 }
 
@@ -192,7 +196,7 @@ __device__ __forceinline__ uint32_t load_pair(const uint16_t* p, uint32_t l, uin
 // thread is sm[slot * STRIDE + tid] for slots [0, S_WORDS). nwords_out: the part's word count
 // (0: the part lies past the last row and root is the public 0).
 template <int MODE, int STRIDE>
-__device__ __forceinline__ void part_root(const CmpParams& P, uint32_t n, uint32_t blk, uint32_t part, uint32_t ks,
+__device__ __forceinline__ void part_root(const CmpParams& P, const Seeds& sd, uint32_t n, uint32_t blk, uint32_t part, uint32_t ks,
                                           uint32_t* sm, uint32_t tid, B3& root, uint32_t& nwords_out) {
   auto S = [&](int slot) -> uint32_t& { return sm[slot * STRIDE + tid]; };
   const uint32_t req = P.col_tags[2 * n], tag = P.col_tags[2 * n + 1];
@@ -268,7 +272,7 @@ __device__ __forceinline__ void part_root(const CmpParams& P, uint32_t n, uint32
         for (int v = 0; v < 32; ++v) S(S_X + 32 * j + v) = a[v];
       }
       GateRng fa{static_cast<uint32_t>(grow >> 5), tag, req, {}}, rc{static_cast<uint32_t>(grow >> 5), tag, req, {}};
-      bit_extract<31, MSB_GATE0>(P.seeds, fa, rc, [&](int j, int b) -> uint32_t { return S(S_X + 32 * j + b); }, msb,
+      bit_extract<31, MSB_GATE0>(sd, fa, rc, [&](int j, int b) -> uint32_t { return S(S_X + 32 * j + b); }, msb,
                                  b30);
     } else if constexpr (MODE == MODE_PLAIN) {
       // ---- v = t - dot, t = floor(a ml / 2^16) public (component 0); bit-slice; MSB of 16 bits ----
@@ -290,7 +294,7 @@ __device__ __forceinline__ void part_root(const CmpParams& P, uint32_t n, uint32
         for (int v = 0; v < 16; ++v) S(S_X + 32 * j + v) = a[v];
       }
       GateRng fa{static_cast<uint32_t>(grow >> 5), tag, req, {}}, rc{static_cast<uint32_t>(grow >> 5), tag, req, {}};
-      bit_extract<15, 0>(P.seeds, fa, rc, [&](int j, int b) -> uint32_t { return S(S_X + 32 * j + b); }, msb, b30);
+      bit_extract<15, 0>(sd, fa, rc, [&](int j, int b) -> uint32_t { return S(S_X + 32 * j + b); }, msb, b30);
     } else {
       // ---- ShareSplit of ml: bit-slice each component (bits 0..15); keep its raw pairs ----
 #pragma unroll
@@ -316,7 +320,7 @@ __device__ __forceinline__ void part_root(const CmpParams& P, uint32_t n, uint32
       GateRng fa{static_cast<uint32_t>(grow >> 5), tag, req, {}}, rc{static_cast<uint32_t>(grow >> 5), tag, req, {}};
       B3 r17, r16;
       bit_extract<17, LIFT_GATE0>(
-          P.seeds, fa, rc, [&](int j, int b) -> uint32_t { return b < 16 ? S(S_X + 32 * j + b) : 0u; }, r17, r16);
+          sd, fa, rc, [&](int j, int b) -> uint32_t { return b < 16 ? S(S_X + 32 * j + b) : 0u; }, r17, r16);
       // ---- per comparison: BitInject (3-party OT), ConstLift, v = a*ml' - 2^16*dot ----
       // Row pair (l, l+1) reads raw ml word 16 + l/2 of each component before writing v to
       // words l and l+1; those overwrite raw words l-16 and l-15 <= l/2 only once they are read.
@@ -337,9 +341,9 @@ __device__ __forceinline__ void part_root(const CmpParams& P, uint32_t n, uint32
         for (uint32_t e = 0; e < 2; ++e) {
           const uint32_t r = l + e;
           const uint64_t g = grow + r;
-          if ((r & 3u) == 0) q0w = philox(static_cast<uint32_t>(g >> 2), tag, req, IPC_D_INJ0 << 24, P.seeds.s[0]);
+          if ((r & 3u) == 0) q0w = philox(static_cast<uint32_t>(g >> 2), tag, req, IPC_D_INJ0 << 24, sd.k[0]);
           const uint32_t inj0 = word_of(q0w, r & 3u);
-          const uint4 w2 = philox(static_cast<uint32_t>(g), tag, req, IPC_D_INJ2 << 24, P.seeds.s[2]);
+          const uint4 w2 = philox(static_cast<uint32_t>(g), tag, req, IPC_D_INJ2 << 24, sd.k[2]);
           uint32_t A[3], Bv[3];
 #pragma unroll
           for (int which = 0; which < 2; ++which) {
@@ -381,7 +385,7 @@ __device__ __forceinline__ void part_root(const CmpParams& P, uint32_t n, uint32
         for (int v = 0; v < 32; ++v) S(S_X + 32 * j + v) = a[v];
       }
       GateRng fa2{static_cast<uint32_t>(grow >> 5), tag, req, {}}, rc2{static_cast<uint32_t>(grow >> 5), tag, req, {}};
-      bit_extract<31, MSB_GATE0>(P.seeds, fa2, rc2, [&](int j, int b) -> uint32_t { return S(S_X + 32 * j + b); },
+      bit_extract<31, MSB_GATE0>(sd, fa2, rc2, [&](int j, int b) -> uint32_t { return S(S_X + 32 * j + b); },
                                  msb, b30);
     }
     // rows past the end (and, with col_rows, rows past the column's limit) are the public 0
@@ -409,7 +413,7 @@ __device__ __forceinline__ void part_root(const CmpParams& P, uint32_t n, uint32
     uint32_t lvl = 0;
     while (lvl < sub_p && (idx & 1u) && (valid_levels >> lvl & 1u)) {
       const B3 left = {S(S_STK + 3 * lvl), S(S_STK + 3 * lvl + 1), S(S_STK + 3 * lvl + 2)};
-      cur = bor(P.seeds, left, cur, static_cast<uint32_t>(idx >> 1), tag, req,
+      cur = bor(sd, left, cur, static_cast<uint32_t>(idx >> 1), tag, req,
                 (IPC_D_OR << 24) | (1u << 16) | (lvl + 1));
       valid_levels &= ~(1u << lvl);
       ++lvl;
@@ -431,7 +435,7 @@ __device__ __forceinline__ void part_root(const CmpParams& P, uint32_t n, uint32
       if (have) {
         if (valid_levels >> lvl & 1u) {
           const B3 left = {S(S_STK + 3 * lvl), S(S_STK + 3 * lvl + 1), S(S_STK + 3 * lvl + 2)};
-          root = bor(P.seeds, left, root, static_cast<uint32_t>(idx >> 1), tag, req,
+          root = bor(sd, left, root, static_cast<uint32_t>(idx >> 1), tag, req,
                      (IPC_D_OR << 24) | (1u << 16) | (lvl + 1));
         }
         idx >>= 1;

@@ -117,6 +117,7 @@ struct FuseParams {
   uint32_t n_ct;           // column tiles of the launch
   uint16_t* z[NPASS];      // z of pass ps, [n_cols][ldz]
   uint64_t seeds[3];       // seeds[j] shared by parties j and j + 1
+  cmp::Seeds keys;         // their round keys
   uint32_t thr_a;
   uint32_t* part_roots;    // [3][n_cols][ld_parts]: OR root of (column, row tile) of the chunk
   uint64_t ld_parts;
@@ -143,7 +144,6 @@ __device__ __noinline__ void fused_part_compare(const TcParams& p, const FusePar
   for (int j = 0; j < 3; ++j) {
     P.zc[j] = fp.z[2 * j];
     P.zm[j] = fp.z[2 * j + 1];
-    P.seeds.s[j] = fp.seeds[j];
   }
   P.ldz = p.ldz;
   P.n_cols = p.n_cols;
@@ -154,7 +154,7 @@ __device__ __noinline__ void fused_part_compare(const TcParams& p, const FusePar
   P.p = FUSE_LOG2_BLOCK;
   cmp::B3 root;
   uint32_t nw;
-  cmp::part_root<cmp::MODE_LIFT, DRAIN_THREADS>(P, n, rt >> 3, rt & 7u, 3u, scratch, tid, root, nw);
+  cmp::part_root<cmp::MODE_LIFT, DRAIN_THREADS>(P, fp.keys, n, rt >> 3, rt & 7u, 3u, scratch, tid, root, nw);
   const uint64_t plane = static_cast<uint64_t>(p.n_cols) * fp.ld_parts;
   const uint64_t at = static_cast<uint64_t>(n) * fp.ld_parts + rt;
   fp.part_roots[at] = root.c0;
@@ -561,6 +561,7 @@ int ring_gemm_compare_tc(uint32_t segments, const int8_t* const x_lo[6], const i
   fp.n_ct = (n_cols + 255) / 256;
   for (uint32_t s = 0; s < NPASS; ++s) fp.z[s] = z[s];
   for (int j = 0; j < 3; ++j) fp.seeds[j] = seeds[j];
+  fp.keys = cmp::make_seeds(seeds);
   fp.thr_a = thr_a;
   fp.part_roots = part_roots;
   fp.ld_parts = ld_parts;
