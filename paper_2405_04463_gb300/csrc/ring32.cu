@@ -46,7 +46,7 @@ __device__ __forceinline__ uint16_t f16_of8(int8_t v) { return __half_as_ushort(
 // A0 over Z_{2^32}: one thread per (row, 2 consecutive elements); one Philox call per vector
 // gives both elements' x_0, x_1 (words 2e, 2e + 1).
 __global__ void encode_share32_kernel(const uint64_t* __restrict__ code_bits, const uint64_t* __restrict__ mask_bits,
-                                      uint32_t n, uint32_t l, uint64_t seed, uint32_t side, uint32_t idx0,
+                                      uint32_t n, uint32_t l, const __grid_constant__ PhiloxKey key, uint32_t side, uint32_t idx0,
                                       uint32_t* __restrict__ code_sh, uint32_t* __restrict__ mask_sh) {
   const uint32_t pairs = l >> 1;
   const uint64_t tid = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x;
@@ -60,7 +60,7 @@ __global__ void encode_share32_kernel(const uint64_t* __restrict__ code_bits, co
   const uint64_t at = static_cast<uint64_t>(r) * l + b0;
 #pragma unroll
   for (uint32_t vec = 0; vec < 2; ++vec) {
-    const uint4 w = philox(t, idx0 + r, (side << 8) | vec, IPC_D_SHARE32 << 24, seed);
+    const uint4 w = philox(t, idx0 + r, (side << 8) | vec, IPC_D_SHARE32 << 24, key);
     uint32_t x0[2] = {w.x, w.z}, x1[2] = {w.y, w.w}, x2[2];
 #pragma unroll
     for (uint32_t e = 0; e < 2; ++e) {
@@ -692,7 +692,7 @@ extern "C" int ipc_encode_share32(const uint64_t* code_bits, const uint64_t* mas
   const uint64_t total = static_cast<uint64_t>(n) * (l / 2);
   const uint32_t bs = 256;
   encode_share32_kernel<<<static_cast<unsigned>((total + bs - 1) / bs), bs, 0, static_cast<cudaStream_t>(stream)>>>(
-      code_bits, mask_bits, n, l, client_seed, side, idx0, code_sh, mask_sh);
+      code_bits, mask_bits, n, l, philox_key(client_seed), side, idx0, code_sh, mask_sh);
   IPC_CUDA_TRY(cudaGetLastError());
   return IPC_OK;
 }
