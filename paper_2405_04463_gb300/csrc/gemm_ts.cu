@@ -23,8 +23,8 @@
 //
 // Measured (one ring GEMM of l = 12,800, K = 25,600, CUDA events, both forms in turn in one process):
 //   65,536 rows x 992 columns: 5.6-5.8 ms against 6.3-6.6 ms (power cap; 5.4 against 6.1 ms cold);
-//   100,000 rows x 31 columns: 0.86 ms against 2.57 ms (the database bytes at 6.0 TB/s);
-//   1,000 rows x 4 columns: 0.025 ms against 0.43 ms (K split over a cluster);
+//   100,000 rows x 31 columns: 0.87 ms against 2.57 ms (the database bytes at 5.9 TB/s);
+//   1,000 rows x 4 columns: 0.023 ms against 0.43 ms (K split over a cluster);
 //   19,456 rows (one tile per SM): 64 / 128 / 160 / 208 columns 0.17 / 0.25 / 0.31 / 0.37 ms against 0.44-0.48.
 //
 // Roles (one CTA per tile of 128 database rows x tn query columns, 16 warps):
@@ -214,15 +214,20 @@ struct Sched<4> {
 
 // KBS: k-blocks of a widened stage; KQ: of a query stage; KR: elements of K of a raw stage; NA, NQ:
 // widened and query stages; DW, WW: drain and widening warps; MAXG: 16-column groups of a drain thread.
-template <int KBS_, int KQ_, int KR_, uint32_t NA_, uint32_t NQ_, int DW_, int WW_, int MAXG_>
+// PAIR: both limb products of lo in one MMA, its B the lo and hi query tiles one under the other
+// (N = 2 tn) and its D [L | C]; two such accumulator pairs take turns, so no drain is waited for. At
+// 32 columns the MMA warp needs 40-50 cycles to issue an MMA of 16, and this saves one in three:
+// 100,000 rows x 62 columns 0.88 ms against 1.04 ms, 93 columns 1.32 against 1.49 ms.
+template <int KBS_, int KQ_, int KR_, uint32_t NA_, uint32_t NQ_, int DW_, int WW_, int MAXG_, bool PAIR_ = false>
 struct Cfg {
+  static constexpr bool PAIR = PAIR_;
   static constexpr uint32_t KBS = KBS_, KQ = KQ_, KR = KR_, NA = NA_, NQ = NQ_, DW = DW_, WW = WW_, MAXG = MAXG_;
   static constexpr uint32_t THREADS = (ISSUE_WARPS + DW + WW) * 32;
   static constexpr uint32_t RAW_STAGE = 2 * TM * KR;  // lo and hi tiles
   static constexpr uint32_t NUM_BARS = 2 * NQ + 2 * NA + 2 * MAX_NR + 6;
   static constexpr uint32_t q_stage(uint32_t tn) { return KQ * 2 * tn * KB * 2; }
   // the widest tile: its accumulators and widened stages fit the 512 TMEM columns
-  static constexpr uint32_t TN_TMEM = (512 - NA * KBS * A_COLS) / 2, TN_DRAIN = MAXG * 16 * (DW / 4);
+  static constexpr uint32_t TN_TMEM = (512 - NA * KBS * A_COLS) / (PAIR ? 4 : 2), TN_DRAIN = MAXG * 16 * (DW / 4);
   static constexpr uint32_t TN = TN_TMEM < TN_DRAIN ? TN_TMEM : TN_DRAIN;
   static constexpr uint32_t raw_stages(uint32_t tn) {
     const uint32_t n = (SMEM_MAX - 1024 - 8 * NUM_BARS - NQ * q_stage(tn)) / RAW_STAGE;
@@ -234,13 +239,14 @@ struct Cfg {
 };
 // By tile width. Narrow tiles are bound by the database bytes and by the MMA warp's pace per stage: long
 // stages and eight widening warps. From 129 columns on TMEM leaves room for shorter stages only.
-using Cfg64 = Cfg<4, 4, 128, 2, 4, 4, 8, 4>;
+using Cfg64 = Cfg<4, 4, 128, 2, 4, 4, 8, 4, true>;
+using Cfg96 = Cfg<2, 2, 128, 2, 4, 4, 8, 6, true>;
 using Cfg128 = Cfg<2, 2, 128, 4, 4, 4, 8, 8>;
 using Cfg160 = Cfg<2, 2, 128, 3, 3, 4, 8, 10>;
 using Cfg192 = Cfg<1, 2, 64, 3, 3, 8, 4, 6>;
 using Cfg208 = Cfg<1, 2, 64, 3, 3, 8, 4, 7>;
-static_assert(Cfg64::TN >= 64 && Cfg128::TN >= 128 && Cfg160::TN >= 160 && Cfg192::TN >= 192 && Cfg208::TN >= MAX_TN, "");
-static_assert(Cfg64::raw_stages(64) >= 2 && Cfg128::raw_stages(128) >= 2 && Cfg160::raw_stages(160) >= 2 &&
+static_assert(Cfg64::TN >= 64 && Cfg96::TN >= 96 && Cfg128::TN >= 128 && Cfg160::TN >= 160 && Cfg192::TN >= 192 && Cfg208::TN >= MAX_TN, "");
+static_assert(Cfg64::raw_stages(64) >= 2 && Cfg96::raw_stages(96) >= 2 && Cfg128::raw_stages(128) >= 2 && Cfg160::raw_stages(160) >= 2 &&
                   Cfg192::raw_stages(192) >= 2 && Cfg208::raw_stages(208) >= 2,
               "raw copies run ahead of the widening");
 
@@ -365,7 +371,8 @@ __global__ void __launch_bounds__(F::THREADS, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = s_tmem;
-  const uint32_t tL = tmem, tC = tmem + tn, tA = tmem + 2 * tn;
+  // PAIR: accumulator pair b at 2 tn b, its full and empty barriers in c_full, c_empty (b = 0) and l_full, l_empty
+  const uint32_t tL = tmem, tC = tmem + tn, tA = tmem + (F::PAIR ? 4 : 2) * tn;
   // a wait by the whole warp, which stays converged
   auto all_wait = [&](uint32_t bar, uint32_t par) {
     return __all_sync(0xFFFFFFFFu, mbar_wait(bar, par, p.status, abort)) != 0;
@@ -476,7 +483,37 @@ __global__ void __launch_bounds__(F::THREADS, 1)
       coords(i, q0, d0, ps, nw);
       idesc = (1u << 4) | ((nw >> 3) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
       bool seen = false;
-      for (uint32_t s = 0; s < nst && ok;) {
+      if constexpr (F::PAIR) {
+        const uint32_t idesc1 = (1u << 4) | ((tn >> 3) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
+        const uint32_t idesc2 = (1u << 4) | ((tn >> 2) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
+        for (uint32_t s = 0; s < nst; ++s) {
+          const bool opens = s % CPS == 0;
+          if (opens) {
+            if (!(ok = all_wait(c_per & 1u ? l_empty : c_empty, ((c_per >> 1) & 1u) ^ 1u))) break;
+            ++c_per;
+          }
+          const uint32_t G = i * nst + s, qs = stage_of<NQ>(G / SPQ), as = stage_of<NA>(G);
+          const uint32_t full = c_per & 1u ? c_full : l_full, d = tmem + ((c_per - 1) & 1u) * 2 * tn;
+          if (!seen && !(ok = wait_stage(G))) break;
+          fence_after();
+          const bool next = s + 1 < nst && mbar_try(a_full + 8 * stage_of<NA>(G + 1), phase_of<NA>(G + 1));
+          const uint32_t qb = qring + qs * q_stage, ab = tA + as * (KBS * A_COLS), t0 = G % SPQ * (2 * KBS);
+          if (elect_one()) {
+#pragma unroll
+            for (uint32_t t = 0; t < 2 * KBS; ++t) {
+              const uint32_t b = qb + ((t0 + t) >> 2) * q_blk + ((t0 + t) & 3u) * 32u, a = ab + (t >> 1) * A_COLS + (t & 1u) * 8u;
+              umma_ts(d, a, sdesc128(b), idesc2, !(opens && t == 0));  // lo * [lo' | hi']
+              umma_ts(d + tn, a + 16, sdesc128(b), idesc1, true);      // hi * lo'
+            }
+            if (G % SPQ == SPQ - 1) umma_commit(q_empty + 8 * qs);
+            umma_commit(a_empty + 8 * as);
+            if ((s + 1) % CPS == 0 || s + 1 == nst) umma_commit(full);
+          }
+          __syncwarp();
+          seen = __all_sync(0xFFFFFFFFu, next) != 0;
+        }
+      }
+      for (uint32_t s = F::PAIR ? nst : 0; s < nst && ok;) {
         const bool c_opens = s % CPS == 0, l_opens = s == 0 || s % LPS == LOFF;
         const uint32_t lead = nst - s < LEAD ? nst - s : LEAD, G = i * nst + s;
         if (c_opens && !l_opens) {
@@ -645,7 +682,33 @@ __global__ void __launch_bounds__(F::THREADS, 1)
         if (ng == 0 && lane == 0) mbar_arrive(empty);
         return true;
       };
-      for (uint32_t s = 1; s <= nst && ok; ++s) {
+      if constexpr (F::PAIR) {
+        for (uint32_t s = 0; s < nst; s += CPS, ++c_per) {
+          const uint32_t b = c_per & 1u, d = tmem + lane_base + b * 2 * tn + col0;
+          if (!(ok = all_wait(b ? l_full : c_full, (c_per >> 1) & 1u))) break;
+          fence_after();
+#pragma unroll
+          for (uint32_t gr = 0; gr < MAXG; ++gr) {
+            if (gr < ng) {
+              uint32_t u[16], v[16];
+              tmem_ld16(d + 16 * gr, u);
+              tmem_ld16(d + tn + 16 * gr, v);
+              tmem_wait_ld();
+              if (gr == ng - 1) {  // the last of this warp's columns is in registers
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(b ? l_empty : c_empty);
+              }
+#pragma unroll
+              for (int k = 0; k < 8; ++k)
+                z2[8 * gr + k] = add16x2(z2[8 * gr + k], add16x2(low16x2<1>(u[2 * k], u[2 * k + 1]),
+                                                                 low16x2<256>(v[2 * k], v[2 * k + 1])));
+            }
+          }
+          if (ng == 0 && lane == 0) mbar_arrive(b ? l_empty : c_empty);
+        }
+      }
+      for (uint32_t s = F::PAIR ? nst + 1 : 1; s <= nst && ok; ++s) {
         if (s % CPS == 0 || s == nst) ok = drain(c_full, c_per++ & 1u, tC, c_empty, true);
         if (ok && (s % LPS == LOFF || s == nst)) ok = drain(l_full, l_per++ & 1u, tL, l_empty, false);
       }
@@ -713,6 +776,29 @@ cudaError_t ready() {
   return e;
 }
 
+// CTAs that run at once in clusters of k (one a SM; clusters do not reach every SM), by device.
+constexpr uint32_t MAX_SPLIT = 8;
+uint32_t g_at_once[64][MAX_SPLIT + 1];
+
+cudaError_t clusters_at_once(uint32_t k) {
+  int dev = 0, n = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || dev < 0 || dev >= 64) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(k);
+  cfg.blockDim = dim3(Cfg208::THREADS);
+  cfg.dynamicSmemBytes = SMEM_MAX;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = k;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  e = cudaOccupancyMaxActiveClusters(&n, gemm_ts_kernel<Cfg208, false, true>, &cfg);
+  g_at_once[dev][k] = e == cudaSuccess ? static_cast<uint32_t>(n) * k : 0;
+  return e;
+}
+
 template <class F>
 int launch_ts(const TsMaps& m, TsParams& p, uint32_t ctas, uint32_t split, cudaStream_t stream) {
   p.nr = F::raw_stages(p.tn);
@@ -737,19 +823,23 @@ uint32_t cdiv(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
 
 // Column tiles per row tile and the parts of K (a cluster's CTAs): the pair with the shortest estimate
 //     rounds of the chip x (k-blocks of a CTA x (250 + 2.45 tile columns) + a tile's start and end)
-// in cycles. The cost of a k-block is a line through the measured 1,600 rows x SMs launches (330 cycles at
-// 32 columns, 410 at 64, 490 at 128, 600 at 160, 760 at 208). A few rounds count whole; over many, other
-// launches and drifting tiles fill the last one. Clusters do not reach every SM (about nine in ten).
-// At 1,000 rows x 4 columns splitting K by 8 gives 0.025 ms against 0.15 ms unsplit, at 9,973 x 217 (two
-// tiles of 112, by 2) 0.31 against 0.40 ms; 40,000 x 279 takes two tiles of 144 (0.67 ms; three of 96: 0.73).
+// in cycles. The cost of a k-block is a line through launches of one tile per SM (330 cycles at 32 columns,
+// 410 at 64, 490 at 128, 600 at 160, 760 at 208). A few rounds count whole; over many, other launches and
+// drifting tiles fill the last one.
+// At 1,000 rows x 4 columns splitting K by 8 gives 0.023 ms against 0.15 ms unsplit, at 1,000 x 279 0.042
+// against 0.085 ms with a guess of nine SMs in ten for clusters; 9,973 x 217 takes two tiles of 112 by 2
+// (0.31 ms; unsplit 0.40), 40,000 x 279 two tiles of 144 (0.67 ms; three of 96: 0.73).
 void pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t n_pass, uint32_t kb_total, uint32_t sms, uint32_t& n_ct,
                 uint32_t& split) {
+  int dev = 0;
+  const uint32_t* at_once = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_at_once[dev] : nullptr;
   const uint32_t units = cdiv(n_cols, 16), least = cdiv(units, MAX_TN / 16);
   double best = 1e300;
   for (uint32_t t = least; t <= least + 2 && t <= units; ++t) {
     const double kb_cycles = 250 + 2.45 * 16 * cdiv(units, t), ctas = static_cast<double>(n_pass) * t * row_tiles;
-    for (uint32_t s = 1; s <= 8 && s <= kb_total / KB_UNIT; ++s) {
-      const double rounds = ctas * s / (s == 1 ? sms : std::max(1u, sms * 9 / 10 / s) * s);
+    for (uint32_t s = 1; s <= MAX_SPLIT && s <= kb_total / KB_UNIT; ++s) {
+      if (s > 1 && (!at_once || at_once[s] == 0)) continue;
+      const double rounds = ctas * s / (s == 1 ? sms : at_once[s]);
       const double cost = (rounds < 4 ? std::ceil(rounds) : rounds + 0.5) * (kb_cycles * kb_total / s + (s == 1 ? 10000 : 14000));
       if (cost < best * 0.999) {
         best = cost;
@@ -782,10 +872,12 @@ int ring_gemm_ts_group(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32
   static PerDevice attr;
   IPC_CUDA_TRY(attr.run([] {
     cudaError_t e = ready<Cfg64>();
+    if (e == cudaSuccess) e = ready<Cfg96>();
     if (e == cudaSuccess) e = ready<Cfg128>();
     if (e == cudaSuccess) e = ready<Cfg160>();
     if (e == cudaSuccess) e = ready<Cfg192>();
     if (e == cudaSuccess) e = ready<Cfg208>();
+    for (uint32_t k = 2; k <= MAX_SPLIT && e == cudaSuccess; ++k) e = clusters_at_once(k);
     return e;
   }));
   TsParams p{};
@@ -807,6 +899,7 @@ int ring_gemm_ts_group(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32
     p.tn = 16 * cdiv(cdiv(n_cols, 16), p.n_col_tiles);
   }
   const uint32_t raw_cols = p.tn <= 64    ? Cfg64::KR
+                            : p.tn <= 96  ? Cfg96::KR
                             : p.tn <= 128 ? Cfg128::KR
                             : p.tn <= 160 ? Cfg160::KR
                             : p.tn <= 192 ? Cfg192::KR
@@ -859,6 +952,7 @@ int ring_gemm_ts_group(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32
   p.status = status_ptr();
   const uint32_t ctas = col_tiles ? sms : n_pass * p.n_col_tiles * p.n_row_tiles * split;
   if (p.tn <= 64) return launch_ts<Cfg64>(m, p, ctas, split, stream);
+  if (p.tn <= 96) return launch_ts<Cfg96>(m, p, ctas, split, stream);
   if (p.tn <= 128) return launch_ts<Cfg128>(m, p, ctas, split, stream);
   if (p.tn <= 160) return launch_ts<Cfg160>(m, p, ctas, split, stream);
   if (p.tn <= 192) return launch_ts<Cfg192>(m, p, ctas, split, stream);
