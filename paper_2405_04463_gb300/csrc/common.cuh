@@ -18,7 +18,9 @@ namespace ipc {
 // ---------------------------------------------------------------------------
 // The round keys of a seed. Kernels that draw many blocks take them as launch parameters: a round is
 // then two wide products and two three-input xors with the key as a constant-bank operand, four
-// instructions where advancing the key costs two more.
+// instructions where advancing the key costs two more. Kernels that draw a few in their epilogue take the
+// seed and advance the key: twenty keys derived there are kept in registers across the main loop (integer
+// step of 8,000 rows x 248 columns: 9.46 against 9.16 ms).
 struct PhiloxKey {
   uint32_t k[20];
 };
@@ -46,7 +48,19 @@ __device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, u
 }
 
 __device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint64_t seed) {
-  return philox(c0, c1, c2, c3, philox_key(seed));
+  uint32_t k0 = static_cast<uint32_t>(seed), k1 = static_cast<uint32_t>(seed >> 32);
+#pragma unroll
+  for (int r = 0; r < 10; ++r) {
+    const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
+    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
+    c0 = hi1 ^ c1 ^ k0;
+    c2 = hi0 ^ c3 ^ k1;
+    c1 = lo1;
+    c3 = lo0;
+    k0 += 0x9E3779B9u;
+    k1 += 0xBB67AE85u;
+  }
+  return make_uint4(c0, c1, c2, c3);
 }
 
 __device__ __forceinline__ uint32_t word_of(const uint4& w, uint32_t i) {
