@@ -218,11 +218,11 @@ int ipc_ring_gemm_tiles(int variant, const int8_t* const x_lo[2], const int8_t* 
  * integer paths (ipc_split_limbs; x planes [x_rows][l], the size of the u16
  * shares); the query operand comes from ipc_prep_query_f16 (fp16 bit patterns
  * of the int8 limbs, b planes [n_pad][2l]). Each k-block of the database tile is
- * widened from int8 to fp16 in shared memory inside the kernel. The products run
- * as fp16 MMAs with fp32 accumulators in tensor memory; each accumulator is
- * drained and restarts at 1.5 * 2^23 after at most 256 products, so all partial
- * sums stay integers inside [2^23, 2^24], where fp32 addition is exact, and the
- * result is bit-identical to the integer paths.
+ * widened from int8 to fp16 into tensor memory inside the kernel. The products
+ * run as fp16 MMAs with fp32 accumulators in tensor memory; each accumulator
+ * starts at 0 and is drained after at most 1,024 products of at most 2^14, so
+ * all partial sums are integers of at most 2^24, where fp32 addition is exact,
+ * and the result is bit-identical to the integer paths.
  * Arguments, alignment rules and errors as ipc_ring_gemm.
  */
 int ipc_ring_gemm_tc(const int8_t* const x_lo[2], const int8_t* const x_hi[2], size_t x_rows,

@@ -488,10 +488,11 @@ extern "C" int submit_queries(ipc_ctx* c, const uint16_t* const code[3], const u
   auto i8p = [](const uint8_t* p) { return reinterpret_cast<const int8_t*>(p); };
   auto cf16 = [](const uint8_t* p) { return reinterpret_cast<const uint16_t*>(p); };
   const bool fused = c->cfg.fused != 0;
-  // tcgen05 paths with every vector over Z_2^16: the three parties' GEMMs are launched together, on one
-  // stream. Chunks on two streams put two query operands in L2 at once: 64.6 against 62.3 ms a step of
-  // 100,000 rows x 992 columns.
-  const bool joint = !fused && c->qsz == 2 && !c->cfg.lift;
+  // tcgen05 paths: the three parties' Z_2^16 GEMMs are launched together, on one stream. Chunks on two
+  // streams put two query operands in L2 at once: 64.6 against 62.3 ms a step of 100,000 rows x 992
+  // columns. The Z_2^32 GEMMs go on the party streams, where each fills the last round of the one before:
+  // 20.6 against 21.3 ms a ConstLift step of 30,000 x 496 on one stream.
+  const bool joint = !fused && c->qsz == 2;
   if (joint) {
     for (int i = 1; i < 3; ++i) {
       SUB_TRY(cudaEventRecord(c->ev_gemm[i][0], c->sp[i]));
@@ -554,11 +555,27 @@ extern "C" int submit_queries(ipc_ctx* c, const uint16_t* const code[3], const u
       // seeds make its zero share vanish
       RingGemm g[RING_GEMM_PASSES];
       uint32_t n_pass = 0;
+      for (int i = 0; i < (c->cfg.lift ? 3 : 1); ++i) SUB_TRY(cudaStreamWaitEvent(c->sp[i], c->ev_cmp[set], 0));
       for (int vec = 0; vec < 2; ++vec)
         for (int i = 0; i < 3; ++i) {
           const bool clear = plain && vec == 1;
           if (clear && i != 0) continue;
           const int prev = (i + 2) % 3, other = clear || c->cfg.path == IPC_PATH_TCG ? i : prev;
+          uint8_t* zo = vec == 0 ? zc[i] : zm[i];
+          if (wide(c, vec)) {
+            // lifting variants: the ring product over Z_2^32, four limbs, K = 2l
+            const int8_t* x8[8];
+            const uint16_t* b4[4];
+            for (int t = 0; t < 4; ++t) {
+              x8[t] = i8p(plane(c, ch, i, vec, t));
+              x8[4 + t] = i8p(plane(c, ch, prev, vec, t));
+              b4[t] = cf16(bq(i, vec, t));
+            }
+            SUB_RC(ring_gemm_tc32(2, x8, ch.rows, b4, N, n_pad, l, sl.tags, c->cfg.seeds[i], c->cfg.seeds[prev],
+                                  static_cast<uint32_t>(vec), reinterpret_cast<uint32_t*>(zo), ldz, ch.row0,
+                                  c->sp[i]));
+            continue;
+          }
           g[n_pass++] = RingGemm{{i8p(plane(c, ch, i, vec, 0)), i8p(plane(c, ch, other, vec, 0))},
                                  {i8p(plane(c, ch, i, vec, 1)), i8p(plane(c, ch, other, vec, 1))},
                                  other == i ? 1u : 2u,
@@ -567,42 +584,25 @@ extern "C" int submit_queries(ipc_ctx* c, const uint16_t* const code[3], const u
                                  c->cfg.seeds[i],
                                  c->cfg.seeds[clear ? i : prev],
                                  static_cast<uint32_t>(vec),
-                                 reinterpret_cast<uint16_t*>(vec == 0 ? zc[i] : zm[i])};
+                                 reinterpret_cast<uint16_t*>(zo)};
         }
-      SUB_TRY(cudaStreamWaitEvent(c->sp[0], c->ev_cmp[set], 0));
-      SUB_RC(ring_gemm_ts(n_pass, g, ch.rows, N, n_pad, l, sl.tags, ldz, ch.row0, 0, nullptr, nullptr, c->sp[0]));
-      SUB_TRY(cudaEventRecord(c->ev_gemm[0][set], c->sp[0]));
-      SUB_TRY(cudaStreamWaitEvent(c->sc, c->ev_gemm[0][set], 0));
+      if (n_pass > 0)
+        SUB_RC(ring_gemm_ts(n_pass, g, ch.rows, N, n_pad, l, sl.tags, ldz, ch.row0, 0, nullptr, nullptr, c->sp[0]));
+      for (int i = 0; i < (c->cfg.lift ? 3 : 1); ++i) {
+        SUB_TRY(cudaEventRecord(c->ev_gemm[i][set], c->sp[i]));
+        SUB_TRY(cudaStreamWaitEvent(c->sc, c->ev_gemm[i][set], 0));
+      }
     }
     for (int i = 0; i < 3 && !joint; ++i) {
       const int prev = (i + 2) % 3;
       SUB_TRY(cudaStreamWaitEvent(c->sp[i], c->ev_cmp[set], 0));
       for (int vec = 0; vec < 2; ++vec) {
         uint16_t* zo = reinterpret_cast<uint16_t*>(vec == 0 ? zc[i] : zm[i]);
-        if (wide(c, vec)) {
-          // lifting variants: the ring product over Z_2^32, four limbs, K = 2l
-          const int8_t* x8[8];
-          const uint16_t* b4[4];
-          for (int t = 0; t < 4; ++t) {
-            x8[t] = i8p(plane(c, ch, i, vec, t));
-            x8[4 + t] = i8p(plane(c, ch, prev, vec, t));
-            b4[t] = cf16(bq(i, vec, t));
-          }
-          SUB_RC(ring_gemm_tc32(2, x8, ch.rows, b4, N, n_pad, l, sl.tags, c->cfg.seeds[i], c->cfg.seeds[prev],
-                                static_cast<uint32_t>(vec), reinterpret_cast<uint32_t*>(zo), ldz, ch.row0, c->sp[i]));
-        } else if (c->cfg.path == IPC_PATH_TC) {  // ConstLift's code vector
-          const int8_t* xl[2] = {i8p(plane(c, ch, i, vec, 0)), i8p(plane(c, ch, prev, vec, 0))};
-          const int8_t* xh[2] = {i8p(plane(c, ch, i, vec, 1)), i8p(plane(c, ch, prev, vec, 1))};
-          SUB_RC(ipc_ring_gemm_tc(xl, xh, ch.rows, cf16(bq(i, vec, 0)), cf16(bq(i, vec, 1)), N, n_pad, l, sl.tags,
-                                  c->cfg.seeds[i], c->cfg.seeds[prev], static_cast<uint32_t>(vec), zo, ldz, ch.row0,
-                                  c->sp[i]));
-        } else {
-          const int8_t* xl[2] = {i8p(plane(c, ch, i, vec, 0)), i8p(plane(c, ch, prev, vec, 0))};
-          const int8_t* xh[2] = {i8p(plane(c, ch, i, vec, 1)), i8p(plane(c, ch, prev, vec, 1))};
-          SUB_RC(ipc_ring_gemm(c->cfg.path, xl, xh, ch.rows, i8p(bq(i, vec, 0)), i8p(bq(i, vec, 1)), N, n_pad, l,
-                               sl.tags, c->cfg.seeds[i], c->cfg.seeds[prev], static_cast<uint32_t>(vec), zo, ldz,
-                               ch.row0, c->sp[i]));
-        }
+        const int8_t* xl[2] = {i8p(plane(c, ch, i, vec, 0)), i8p(plane(c, ch, prev, vec, 0))};
+        const int8_t* xh[2] = {i8p(plane(c, ch, i, vec, 1)), i8p(plane(c, ch, prev, vec, 1))};
+        SUB_RC(ipc_ring_gemm(c->cfg.path, xl, xh, ch.rows, i8p(bq(i, vec, 0)), i8p(bq(i, vec, 1)), N, n_pad, l,
+                             sl.tags, c->cfg.seeds[i], c->cfg.seeds[prev], static_cast<uint32_t>(vec), zo, ldz,
+                             ch.row0, c->sp[i]));
       }
       SUB_TRY(cudaEventRecord(c->ev_gemm[i][set], c->sp[i]));
       SUB_TRY(cudaStreamWaitEvent(c->sc, c->ev_gemm[i][set], 0));

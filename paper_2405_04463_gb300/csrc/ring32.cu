@@ -8,23 +8,16 @@
 // A3 (gemm_tc32_kernel): the ring dot product on tcgen05 with fp32 TMEM accumulators, exact:
 //     z = sum_s 2^(8s) S_s (mod 2^32),  S_s = sum over a + b = s of sum_k x_a[k] y_b[k],
 //   ten limb products per k (1 + 2 + 3 + 4 for s = 0..3); products with a + b > 3 vanish mod
-//   2^32. Each S_s is accumulated in a TMEM accumulator started at M = 1.5 * 2^23 and drained
-//   while every partial sum stays within M +- 2^22 (so every fp32 addition is exact, as in the
-//   16-bit kernel): S_s gains at most (s + 1) 2^14 per k, so S_3 and S_2 are drained every 64 k,
-//   S_1 every 128 k, S_0 every 256 k. Two passes per tile (S_3 and S_2, then S_1 and S_0) share
-//   the 512 TMEM columns; a drain adds the raw bits, shifted by 8s, to running sums: mod 2^16
-//   for (S_2 + 2^8 S_3), whose bits(M) terms vanish, and mod 2^32 for S_0 + 2^8 S_1, whose
-//   bits(M) terms are subtracted once, up front. The database limbs are widened from int8 to
-//   fp16 in shared memory, as in the 16-bit kernel. Every wait is bounded (2 s, or sooner once
-//   another role has failed); a failed CTA raises the status word, lets its copies and MMAs
-//   finish and frees its tensor memory.
+//   2^32. The database limbs are widened from int8 to fp16 on their way into tensor memory.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+#include <cmath>
 #include <mutex>
 #include <string>
 #include <type_traits>
 
-#include "tcgen05.cuh"
+#include "tcgen05_ts.cuh"
 
 namespace ipc {
 namespace {
@@ -158,453 +151,490 @@ __global__ void prep_query32_kernel(const uint32_t* __restrict__ y, uint64_t pla
 }
 
 // ----------------------------------- A3 -----------------------------------
-// One CTA per tile of 128 database rows x 256 query columns (MMA 128 x 256 x 16). Four 256-column
-// accumulators would need 1,024 TMEM columns (an SM has 512), so the tile runs in two passes of
-// two accumulators each, over the same rings:
-//   pass A (stages 0 .. KBT-1, one k-block each): S_3 and S_2, seven limb products over limbs
-//     0-3. Only U = (S_2 + 2^8 S_3) mod 2^16 matters (it enters z shifted by 16), so its running
-//     sums are kept mod 2^16, two columns to a register; at the end of the pass they go to z as
-//     U << 16 (global memory, read back by the epilogue).
-//   pass B (stages KBT .. KBT + KBT/2 - 1, two k-blocks each): S_1 and S_0, three limb products
-//     over limbs 0-1, whose sums are kept mod 2^32.
-// A stage holds four tiles of each operand: limbs 0-3 of one k-block (pass A) or limbs 0-1 of
-// two k-blocks (pass B), so the rings run on from one pass into the other.
-constexpr int TM = 128, TN = 256, KB = 32, SLOTS = 4;
-constexpr int W_TILE = TM * KB * 2;  // 8 KiB widened (fp16) database tile
-constexpr int RAW_TILE = TM * KB;    // 4 KiB raw (int8) database tile
-constexpr int B_TILE = TN * KB * 2;  // 16 KiB query tile
-constexpr int QS = 2, WS = 2, RS = 2;  // stages of the query, widened and raw rings
-constexpr int Q_STAGE = SLOTS * B_TILE;    // 64 KiB
-constexpr int W_STAGE = SLOTS * W_TILE;    // 32 KiB
-constexpr int R_STAGE = SLOTS * RAW_TILE;  // 16 KiB
-constexpr int W_OFF = QS * Q_STAGE, R_OFF = W_OFF + WS * W_STAGE, BAR_OFF = R_OFF + RS * R_STAGE;
-constexpr int THREADS = 12 * 32, DRAIN_THREADS = 8 * 32;
-constexpr int WIDEN_WARP0 = 2, WIDEN_THREADS = 2 * 32, DRAIN_WARP0 = 4;
-constexpr uint32_t TMEM_COLS = 2 * TN;  // region 0 (S_2, then S_0) and region 1 (S_3, then S_1)
-constexpr uint32_t MAGIC = 0x4B400000u;  // fp32 bits of 1.5 * 2^23
-// q_full[QS], q_empty[QS], w_full[WS], w_empty[WS], r_full[RS], r_empty[RS], a_full[2],
-// a_empty[2], done
-constexpr int NUM_BARS = 2 * QS + 2 * WS + 2 * RS + 5;
-constexpr int SMEM_BYTES = BAR_OFF + 1024 + 8 * NUM_BARS;
-static_assert(SMEM_BYTES <= 232448, "dynamic shared memory per block");
-static_assert(TN * TM * 4 <= QS * Q_STAGE, "the z tile is staged in the Q ring");
-// kind::f16: D f32, A and B f16, both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28
-constexpr uint32_t IDESC = (1u << 4) | (static_cast<uint32_t>(TN >> 3) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
-
-// Drain periods, in stages: pass A drains both regions every 2 stages (64 k: S_3 gains at most
-// 4 * 2^14 per k); pass B drains S_1 every 2 stages (128 k) and S_0 every 4 (256 k).
-// Operand tile t of stage G: its limb and k-block.
-__device__ __forceinline__ void stage_slot(uint32_t G, uint32_t kbt, uint32_t t, uint32_t& limb, uint32_t& kb) {
-  if (G < kbt) {
-    limb = t;
-    kb = G;
-  } else {
-    limb = t & 1u;
-    kb = 2u * (G - kbt) + (t >> 1);
-  }
-}
+// One CTA per tile of 128 database rows x tn query columns. With four balanced limbs per operand
+// z = sum over s of 2^(8s) S_s, S_s the sum of the limb products x_a y_b, a + b = s (ten per k; products
+// with a + b > 3 vanish mod 2^32). The database limbs are widened in registers and stored to tensor
+// memory, as in the 16-bit kernel, and the query tiles of a stage lie one under the other in shared
+// memory, so that one MMA of N = 2 tn multiplies a limb with two of them; its D is a pair of neighbouring
+// accumulators [S_0 | S_1 | S_2 | S_3]:
+//     H:  [S_2 | S_3] += x_0 [y_2 | y_3], x_1 [y_1 | y_2], x_2 [y_0 | y_1];  S_3 += x_3 y_0
+//     Lo: [S_0 | S_1] += x_0 [y_0 | y_1];  S_1 += x_1 y_0
+// Every accumulator starts at 0 and is drained while all partial sums are integers of at most 2^24: H
+// every 256 k (S_3 gains at most 4 * 2^14 per k; only (S_2 + 2^8 S_3) mod 2^16 matters), Lo every 512 k.
+// While H is drained the Lo products of the next stages run, and the other way round.
+// Bound by the MMAs: 5 cycles per k and column, 64 B of query operand per cycle from shared memory. The
+// earlier form kept both operands in shared memory, drained every 64 k and needed two passes over K for
+// tiles of 256 columns, because four accumulators of that width do not fit the 512 TMEM columns; with A
+// in tensor memory narrow MMAs run at the same rate, and 96 columns leave room for two widened k-blocks.
+// 65,536 rows x 992 columns (K = 25,600): 21.6 ms against 22.7 ms; 30,000 x 496: 5.26 against 6.09 ms;
+// 19,456 x 96 (a tile per SM): 0.59 against 1.60 ms; 1,000 x 31: 0.053 against 1.51 ms. Two warps that
+// issue, one for H and one for Lo, take 5.95 ms at 30,000 x 496.
+constexpr int TM = 128, KB = 32;
+constexpr uint32_t KB_UNIT = 4;        // k-blocks in which K is counted out: 128 elements
+constexpr uint32_t HP = 8, LP = 16;    // k-blocks between drains of H and of Lo
+constexpr uint32_t LOFF = 4;           // Lo's drains fall at LOFF + i LP, away from H's
+constexpr uint32_t KR = 64, KBR = 2;   // elements and k-blocks of a raw or query stage
+constexpr uint32_t NQ = 3, MAX_NR = 4;
+constexpr uint32_t RAW_TILE = TM * KR, RAW_STAGE = 4 * RAW_TILE;
+constexpr uint32_t A_COLS = 64;        // TMEM columns of a widened k-block: four limbs of 16 (two fp16 a column)
+constexpr uint32_t SMEM_MAX = 231424;
+constexpr uint32_t MAX_TN = 96, MAX_SPLIT = 8;
+constexpr uint32_t DW = 8, WW = 8, MAXG = 3, ISSUE_WARPS = 4, THREADS = (ISSUE_WARPS + DW + WW) * 32;
+constexpr uint32_t MAX_NA = 3, NUM_BARS = 2 * NQ + 2 * MAX_NA + 2 * MAX_NR + 6;
+static_assert(MAX_TN <= MAXG * 16 * (DW / 4) && WW == 4 * KBR, "a drain thread's columns; a widening group per k-block of a raw stage");
 
 struct Maps32 {
-  CUtensorMap b[4];   // query limbs [n_pad][K], fp16
-  CUtensorMap a0[4];  // database limbs of the first K segment [x_rows][l], int8
-  CUtensorMap a1[4];  // and of the second
+  CUtensorMap b[4];     // query limbs [n_pad][K], fp16
+  CUtensorMap x[2][4];  // database limbs of the two K segments, [x_rows][l] int8
 };
 
 struct Tc32Params {
-  uint32_t n_cols;
-  uint32_t x_rows;
-  uint32_t kb_total;  // K / KB
-  uint32_t kb_half;   // l / KB: k-blocks below it read the first segment's planes
+  uint32_t n_cols, x_rows, tn, nr, n_ct, n_rt;
+  uint32_t segs, kb_seg;  // K segments; k-blocks of one
   const uint32_t* col_tags;
   uint64_t seed_own, seed_prev;
   uint32_t vec;
   uint32_t* z;
-  uint64_t ldz;
-  uint64_t row0;
+  uint64_t ldz, row0;
   uint32_t* status;
 };
 
-// Roles (12 warps), with three rings as in the 16-bit kernel (query, raw database, widened
-// database), so that the widening runs ahead of the MMAs:
-//   warp 0 lane 0  query producer: per stage, four fp16 query tiles (256 x 32, 64-byte swizzle).
-//   warps 2-3      raw copies and widening: a stage's four raw int8 database tiles (copied RS
-//                  stages ahead) become fp16 operand tiles in the W ring.
-//   warp 1 lane 0  MMA issuer: per stage, region 1's products (S_3, or S_1), then region 0's
-//                  (S_2, or S_0), committing a region's full barrier after the last stage of its
-//                  drain period, then the stage's Q and W slots. Region 1 drains while region
-//                  0's products of the same stage run.
-//   warps 4-11     drain: each thread owns one TMEM lane (database row) and 128 columns.
-// Every wait is bounded (2 s, or sooner once another role has failed); a failed CTA raises the
-// status word, lets its copies and MMAs finish and frees its tensor memory (its z tile is then
-// undefined).
-__global__ void __launch_bounds__(THREADS, 1) gemm_tc32_kernel(const __grid_constant__ Maps32 m, const Tc32Params p) {
+// Warps: 0 query copies, 1 MMAs (one elected lane issues), 2 raw copies, 3 joins the query tiles' arrival to
+// the widened stage's barrier, 4-11 drain (a TMEM lane quarter and half of the columns each), 12-19
+// widening. A cluster's CTAs take parts of K (SPLIT) and join their sums through distributed shared memory.
+// Every wait is bounded (2 s, or sooner once another role has failed); a failed CTA raises the status word,
+// lets its copies and MMAs finish, frees its tensor memory and stores nothing.
+template <uint32_t NA, bool SPLIT>
+__global__ void __launch_bounds__(THREADS, 1)
+    gemm_tc32_kernel(const __grid_constant__ Maps32 maps, const __grid_constant__ Tc32Params p) {
+  constexpr uint32_t LEAD = NA, DT = DW * 32;
+  static_assert(HP - LOFF >= LEAD && LOFF >= LEAD && LP % HP == 0 && NQ * KBR >= LEAD, "drains apart");
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ uint32_t s_abort;
+  const uint32_t tn = p.tn, q_tile = tn * 128, q_stage = 4 * q_tile;
+  uint32_t rank = 0, n_rank = 1;
+  if (SPLIT) {
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_rank));
+  }
+  // the tile: bands of up to 8 column tiles, all row tiles of a band before the next
+  constexpr uint32_t kBand = 8;
+  uint32_t q0, d0, nw;
+  {
+    const uint32_t lin = blockIdx.x / n_rank;
+    const uint32_t band = lin / (kBand * p.n_rt), c0 = band * kBand;
+    const uint32_t width = p.n_ct - c0 < kBand ? p.n_ct - c0 : kBand;
+    const uint32_t in_band = lin - band * kBand * p.n_rt, ct = c0 + in_band % width;
+    const uint32_t units = (p.n_cols + 15) / 16, base = units / p.n_ct, rem = units % p.n_ct;
+    q0 = 16 * (ct * base + (ct < rem ? ct : rem));
+    nw = 16 * (base + (ct < rem ? 1 : 0));
+    d0 = in_band / width * TM;
+  }
+  const uint32_t k_units = p.segs * p.kb_seg / KB_UNIT;
+  const uint32_t kb0 = SPLIT ? k_units * rank / n_rank * KB_UNIT : 0;
+  const uint32_t nst = (SPLIT ? k_units * (rank + 1) / n_rank : k_units) * KB_UNIT - kb0;  // stages: one k-block each
+  // two segments are taken in turn, 128 elements each
+  auto k_of = [&](uint32_t kb, uint32_t& seg) {
+    const uint32_t u = kb / KB_UNIT;
+    seg = p.segs == 2 ? u & 1u : 0u;
+    return static_cast<int32_t>(((p.segs == 2 ? u >> 1 : u) * KB_UNIT + kb % KB_UNIT) * KB);
+  };
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const uint32_t qring = smem_addr(smem), wring = qring + W_OFF, rring = qring + R_OFF, bars = qring + BAR_OFF;
-  const uint32_t q_full = bars, q_empty = q_full + 8 * QS, w_full = q_empty + 8 * QS, w_empty = w_full + 8 * WS,
-                 r_full = w_empty + 8 * WS, r_empty = r_full + 8 * RS;
-  const uint32_t a_full = r_empty + 8 * RS, a_empty = a_full + 16, done_bar = a_full + 32;
+  const uint32_t qring = smem_addr(smem), rring = qring + NQ * q_stage, bars = rring + p.nr * RAW_STAGE;
+  const uint32_t q_full = bars, q_empty = q_full + 8 * NQ, a_full = q_empty + 8 * NQ, a_empty = a_full + 8 * NA,
+                 r_full = a_empty + 8 * NA, r_empty = r_full + 8 * MAX_NR, h_full = r_empty + 8 * MAX_NR,
+                 h_empty = h_full + 8, l_full = h_full + 16, l_empty = h_full + 24, done_bar = h_full + 32;
   volatile uint32_t* abort = &s_abort;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t q0 = blockIdx.x * TN, d0 = blockIdx.y * TM;
-  const uint32_t kbt = p.kb_total;           // a multiple of 8: K is a multiple of 256
-  const uint32_t n_stages = kbt + kbt / 2;   // pass A, then pass B
-
+  const uint32_t warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < QS; ++s) {
+    for (uint32_t s = 0; s < NQ; ++s) {
       mbar_init(q_full + 8 * s, 1);
       mbar_init(q_empty + 8 * s, 1);
     }
-    for (int s = 0; s < WS; ++s) {
-      mbar_init(w_full + 8 * s, WIDEN_THREADS / 32);
-      mbar_init(w_empty + 8 * s, 1);
+    for (uint32_t s = 0; s < NA; ++s) {
+      mbar_init(a_full + 8 * s, WW / 2 + 1);
+      mbar_init(a_empty + 8 * s, 1);
     }
-    for (int s = 0; s < RS; ++s) {
+    for (uint32_t s = 0; s < MAX_NR; ++s) {
       mbar_init(r_full + 8 * s, 1);
-      mbar_init(r_empty + 8 * s, WIDEN_THREADS / 32);
+      mbar_init(r_empty + 8 * s, WW);
     }
-    for (int g = 0; g < 2; ++g) {
-      mbar_init(a_full + 8 * g, 1);
-      mbar_init(a_empty + 8 * g, DRAIN_THREADS / 32);
-    }
+    mbar_init(h_full, 1);
+    mbar_init(h_empty, DW);
+    mbar_init(l_full, 1);
+    mbar_init(l_empty, DW);
     mbar_init(done_bar, 1);
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)),
-                 "r"(TMEM_COLS)
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)), "r"(512u)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = s_tmem;
+  const uint32_t tmem = s_tmem, tH = tmem + 2 * tn, tA = tmem + 4 * tn;
+  auto all_wait = [&](uint32_t bar, uint32_t par) {
+    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, par, p.status, abort)) != 0;
+  };
+  // z = sum + r_i for four rows of a column, r_i = F(seed_own) - F(seed_prev) (App. C)
+  auto put_z = [&](uint32_t col, uint32_t r0, const uint4& a) {
+    if (col >= p.n_cols || r0 >= p.x_rows) return;
+    const uint32_t req = p.col_tags[2 * col], tag = p.col_tags[2 * col + 1];
+    const uint32_t grp = static_cast<uint32_t>((p.row0 + r0) >> 2), ctr3 = (IPC_D_ZA32 << 24) | p.vec;
+    const uint4 fo = philox(grp, tag, req, ctr3, p.seed_own);
+    const uint4 fp = philox(grp, tag, req, ctr3, p.seed_prev);
+    const uint4 v = make_uint4(a.x + fo.x - fp.x, a.y + fo.y - fp.y, a.z + fo.z - fp.z, a.w + fo.w - fp.w);
+    uint32_t* dst = p.z + static_cast<uint64_t>(col) * p.ldz + r0;
+    if (r0 + 4 <= p.x_rows) {
+      __stcs(reinterpret_cast<uint4*>(dst), v);  // streamed: z is read by a later kernel, not from L2
+    } else {
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+      for (uint32_t e = 0; e < p.x_rows - r0; ++e) dst[e] = w[e];
+    }
+  };
 
   if (warp == 0) {
-    // ---------------------------- query TMA producer -----------------------------
-    if (lane == 0) {
-      uint32_t issued = 0;
-      for (uint32_t G = 0; G < n_stages; ++G) {
-        const uint32_t s = G % QS;
-        if (!mbar_wait(q_empty + 8 * s, ((G / QS) & 1u) ^ 1u, p.status, abort)) break;
-        const uint32_t full = q_full + 8 * s, base = qring + s * Q_STAGE;
-        mbar_expect_tx(full, Q_STAGE);
+    // ---------------------------- query copies -----------------------------
+    uint32_t issued = 0;
+    for (uint32_t kb = kb0; kb < kb0 + nst; kb += KBR) {
+      const uint32_t qs = stage_of<NQ>(issued);
+      if (!all_wait(q_empty + 8 * qs, phase_of<NQ>(issued) ^ 1u)) break;
+      if (elect_one()) {
+        const uint32_t full = q_full + 8 * qs, base = qring + qs * q_stage;
+        uint32_t seg;
+        const int32_t k = k_of(kb, seg), kx = k + static_cast<int32_t>(seg * p.kb_seg * KB);
+        mbar_expect_tx(full, q_stage);
 #pragma unroll
-        for (uint32_t t = 0; t < SLOTS; ++t) {
-          uint32_t limb, kb;
-          stage_slot(G, kbt, t, limb, kb);
-          tma_load(base + t * B_TILE, &m.b[limb], static_cast<int32_t>(kb * KB), static_cast<int32_t>(q0), full);
-        }
-        issued = G + 1;
+        for (uint32_t t = 0; t < 4; ++t) tma_load(base + t * q_tile, &maps.b[t], kx, static_cast<int32_t>(q0), full);
       }
-      if (*abort) {
-        // copies that may still be in flight land before the CTA goes on (bounded, no abort)
-        for (uint32_t G = issued > QS ? issued - QS : 0; G < issued; ++G)
-          mbar_wait(q_full + 8 * (G % QS), (G / QS) & 1u, p.status, nullptr);
-      }
+      __syncwarp();
+      ++issued;
+    }
+    if (*abort) {
+      // copies that may still be in flight land before the CTA leaves (bounded, no abort)
+      for (uint32_t G = issued > NQ ? issued - NQ : 0; G < issued; ++G)
+        mbar_wait(q_full + 8 * stage_of<NQ>(G), phase_of<NQ>(G), p.status, nullptr);
     }
   } else if (warp == 1) {
     // -------------------------------- MMA issuer --------------------------------
-    if (lane == 0) {
-      const uint32_t t0 = tmem, t1 = tmem + TN;
-      uint32_t started0 = 0, started1 = 0;  // drain periods started per region
-      bool ok = true;
-      for (uint32_t G = 0; G < n_stages && ok; ++G) {
-        const uint32_t s = G % QS;  // QS == WS
-        if (!mbar_wait(q_full + 8 * s, (G / QS) & 1u, p.status, abort) ||
-            !mbar_wait(w_full + 8 * s, (G / WS) & 1u, p.status, abort))
-          break;
-        fence_after();
-        const bool pass_a = G < kbt;
-        const uint32_t j = pass_a ? G : G - kbt;
-        const bool open1 = (j & 1u) == 0, close1 = (j & 1u) == 1;
-        const bool open0 = pass_a ? (j & 1u) == 0 : (j & 3u) == 0;
-        const bool close0 = pass_a ? (j & 1u) == 1 : (j & 3u) == 3;
-        const uint32_t qb = qring + s * Q_STAGE, wb = wring + s * W_STAGE;
-        if (open1) {
-          if (!mbar_wait(a_empty + 8, started1 & 1u, p.status, abort)) break;
-          ++started1;
-          fence_after();
-        }
-        if (pass_a) {
-#pragma unroll
-          for (uint32_t ks = 0; ks < KB / 16; ++ks) {
-            const uint32_t o = 32u * ks;  // 16 fp16 = 32 bytes along K inside the swizzled row
-#pragma unroll
-            for (uint32_t a = 0; a < 4; ++a)  // S_3: x_a y_(3-a)
-              umma(t1, sdesc(wb + a * W_TILE + o), sdesc(qb + (3 - a) * B_TILE + o), IDESC);
-          }
-        } else {
-#pragma unroll
-          for (uint32_t sub = 0; sub < 2; ++sub)
-#pragma unroll
-            for (uint32_t ks = 0; ks < KB / 16; ++ks) {
-              const uint32_t o = 32u * ks, w = wb + 2 * sub * W_TILE + o, q = qb + 2 * sub * B_TILE + o;
-              umma(t1, sdesc(w), sdesc(q + B_TILE), IDESC);  // S_1: x_0 y_1
-              umma(t1, sdesc(w + W_TILE), sdesc(q), IDESC);  //      x_1 y_0
-            }
-        }
-        if (close1) umma_commit(a_full + 8);
-        if (open0) {
-          if (!mbar_wait(a_empty, started0 & 1u, p.status, abort)) {
-            ok = false;
-            break;
-          }
-          ++started0;
-          fence_after();
-        }
-        if (pass_a) {
-#pragma unroll
-          for (uint32_t ks = 0; ks < KB / 16; ++ks) {
-            const uint32_t o = 32u * ks;
-#pragma unroll
-            for (uint32_t a = 0; a < 3; ++a)  // S_2: x_a y_(2-a)
-              umma(t0, sdesc(wb + a * W_TILE + o), sdesc(qb + (2 - a) * B_TILE + o), IDESC);
-          }
-        } else {
-#pragma unroll
-          for (uint32_t sub = 0; sub < 2; ++sub)
-#pragma unroll
-            for (uint32_t ks = 0; ks < KB / 16; ++ks) {
-              const uint32_t o = 32u * ks;  // S_0: x_0 y_0
-              umma(t0, sdesc(wb + 2 * sub * W_TILE + o), sdesc(qb + 2 * sub * B_TILE + o), IDESC);
-            }
-        }
-        if (close0) umma_commit(a_full);
-        // both slots free once these (and all earlier) MMAs are done
-        umma_commit(q_empty + 8 * s);
-        umma_commit(w_empty + 8 * s);
-      }
-      // every MMA issued above completes before the tensor memory is freed
-      umma_commit(done_bar);
-      mbar_wait(done_bar, 0, p.status, nullptr);
-    }
-  } else if (warp < DRAIN_WARP0) {
-    // ------------------------- raw copies and widening ---------------------------
-    const uint32_t ct = threadIdx.x - WIDEN_WARP0 * 32;
-    uint32_t issued = 0;
-    auto load_raw = [&](uint32_t G) {
-      const uint32_t s = G % RS, full = r_full + 8 * s, base = rring + s * R_STAGE;
-      mbar_expect_tx(full, R_STAGE);
-#pragma unroll
-      for (uint32_t t = 0; t < SLOTS; ++t) {
-        uint32_t limb, kb;
-        stage_slot(G, kbt, t, limb, kb);
-        const bool first = kb < p.kb_half;
-        const int32_t kx = static_cast<int32_t>((first ? kb : kb - p.kb_half) * KB);
-        tma_load(base + t * RAW_TILE, first ? &m.a0[limb] : &m.a1[limb], kx, static_cast<int32_t>(d0), full);
-      }
-      issued = G + 1;
+    const uint32_t id1 = (1u << 4) | ((tn >> 3) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
+    const uint32_t id2 = (1u << 4) | ((tn >> 2) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
+    auto wait_stage = [&](uint32_t G) { return all_wait(a_full + 8 * stage_of<NA>(G), phase_of<NA>(G)); };
+    auto free_stage = [&](uint32_t G) {
+      if (G % KBR == KBR - 1) umma_commit(q_empty + 8 * stage_of<NQ>(G / KBR));
+      umma_commit(a_empty + 8 * stage_of<NA>(G));
     };
-    if (ct == 0)
-      for (uint32_t G = 0; G < n_stages && G < RS; ++G) load_raw(G);
-    uint32_t G = 0;
-    for (; G < n_stages; ++G) {
-      const uint32_t rs = G % RS, ws = G % WS;
-      if (!__all_sync(0xFFFFFFFFu, mbar_wait(r_full + 8 * rs, (G / RS) & 1u, p.status, abort) &&
-                                       mbar_wait(w_empty + 8 * ws, ((G / WS) & 1u) ^ 1u, p.status, abort)))
-        break;
-      widen_tiles<SLOTS, WIDEN_THREADS>(rring + rs * R_STAGE, RAW_TILE, wring + ws * W_STAGE, W_TILE, ct);
-      fence_proxy_async();  // the MMAs read these tiles through the async proxy
+    auto issue_h = [&](uint32_t G, bool frees) {
+      const uint32_t q = qring + stage_of<NQ>(G / KBR) * q_stage + (G % KBR) * 64u, a = tA + stage_of<NA>(G) * A_COLS;
+      const bool opens = G % HP == 0;
+      if (elect_one()) {
+#pragma unroll
+        for (uint32_t ks = 0; ks < KB / 16; ++ks) {
+          const uint32_t b = q + 32u * ks, x = a + 8 * ks;
+          umma_ts(tH, x, sdesc128(b + 2 * q_tile), id2, !(opens && ks == 0));  // x_0 [y_2 | y_3]
+          umma_ts(tH, x + 16, sdesc128(b + q_tile), id2, true);                // x_1 [y_1 | y_2]
+          umma_ts(tH, x + 32, sdesc128(b), id2, true);                         // x_2 [y_0 | y_1]
+          umma_ts(tH + tn, x + 48, sdesc128(b), id1, true);                    // x_3 y_0
+        }
+        if ((G + 1) % HP == 0 || G + 1 == nst) umma_commit(h_full);
+        if (frees) free_stage(G);
+      }
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(w_full + 8 * ws);
-        mbar_arrive(r_empty + 8 * rs);  // this warp has read raw stage rs
-      }
-      if (warp == WIDEN_WARP0 && G + RS < n_stages) {
-        // refill once both warps have read the stage (a bounded wait, warp-uniform like the others)
-        if (!__all_sync(0xFFFFFFFFu, mbar_wait(r_empty + 8 * rs, (G / RS) & 1u, p.status, abort))) break;
-        if (lane == 0) load_raw(G + RS);
-      }
-    }
-    if (ct == 0 && *abort) {
-      // raw copies that may still be in flight land before the CTA leaves (bounded, no abort)
-      for (uint32_t h = G; h < issued; ++h) mbar_wait(r_full + 8 * (h % RS), (h / RS) & 1u, p.status, nullptr);
-    }
-  } else {
-    // ----------------------------------- drain ----------------------------------
-    const uint32_t q = static_cast<uint32_t>(warp) & 3u, h = static_cast<uint32_t>(warp - DRAIN_WARP0) >> 2;
-    const uint32_t tl = tmem + ((32u * q) << 16) + 128u * h;  // region 0; region 1 at + TN
-    const uint32_t row = d0 + 32 * q + lane;
+    };
+    auto issue_l = [&](uint32_t G, bool frees) {
+      const uint32_t q = qring + stage_of<NQ>(G / KBR) * q_stage + (G % KBR) * 64u, a = tA + stage_of<NA>(G) * A_COLS;
+      const bool opens = G == 0 || G % LP == LOFF;
+      if (elect_one()) {
 #pragma unroll
-    for (uint32_t g = 0; g < 4; ++g) {
-      tmem_fill32(tl + 32 * g, MAGIC);
-      tmem_fill32(tl + TN + 32 * g, MAGIC);
-    }
-    tmem_wait_st();
-    fence_before();
-    __syncwarp();
-    if (lane == 0) {
-      mbar_arrive(a_empty);
-      mbar_arrive(a_empty + 8);
-    }
-    uint32_t done0 = 0, done1 = 0;  // drains per region
-    // one drain of a region: wait for its full barrier, hand each 32-column group's fp32 bit
-    // patterns to f, re-base the accumulator, release the region
-    // (W columns a load: 32 in pass A, two loads before each wait; 16 in pass B, one load a wait,
-    // whose 32-bit sums take 128 registers)
-    auto drain = [&](uint32_t region, uint32_t& done, auto&& f, auto width) -> bool {
-      constexpr uint32_t W = decltype(width)::value;
-      if (!__all_sync(0xFFFFFFFFu, mbar_wait(a_full + 8 * region, done & 1u, p.status, abort))) return false;
-      ++done;
-      fence_after();
-      auto ld_ = [&](uint32_t g, uint32_t (&r)[W]) {
-        if constexpr (W == 32) {
-          tmem_ld32(tl + TN * region + W * g, r);
-        } else {
-          tmem_ld16(tl + TN * region + W * g, r);
+        for (uint32_t ks = 0; ks < KB / 16; ++ks) {
+          const uint32_t b = q + 32u * ks, x = a + 8 * ks;
+          umma_ts(tmem, x, sdesc128(b), id2, !(opens && ks == 0));  // x_0 [y_0 | y_1]
+          umma_ts(tmem + tn, x + 16, sdesc128(b), id1, true);       // x_1 y_0
         }
-      };
-      auto fill_ = [&](uint32_t g) {
-        if constexpr (W == 32) {
-          tmem_fill32(tl + TN * region + W * g, MAGIC);
-        } else {
-          tmem_fill16(tl + TN * region + W * g, MAGIC);
+        if (frees) free_stage(G);
+        if ((G + 1) % LP == LOFF || G + 1 == nst) umma_commit(l_full);
+      }
+      __syncwarp();
+    };
+    uint32_t h_per = 0, l_per = 0;
+    bool ok = true;
+    for (uint32_t s = 0; s < nst && ok;) {
+      const bool h_opens = s % HP == 0, l_opens = s == 0 || s % LP == LOFF;
+      const uint32_t lead = nst - s < LEAD ? nst - s : LEAD;
+      if (h_opens && !l_opens) {
+        // the Lo products of the next stages run while H is drained
+        for (uint32_t j = 0; j < lead && ok; ++j) {
+          if (!(ok = wait_stage(s + j))) break;
+          fence_after();
+          issue_l(s + j, false);
         }
-      };
-      if constexpr (W == 32) {
-        // two loads in flight before each wait (pass A: 64 packed sums leave room for them)
-#pragma unroll
-        for (uint32_t g = 0; g < 128 / W; g += 2) {
-          uint32_t r[W], r2[W];
-          ld_(g, r);
-          ld_(g + 1, r2);
-          tmem_wait_ld();
-          f(g, r);
-          f(g + 1, r2);
-          fill_(g);
-          fill_(g + 1);
+        if (!ok || !(ok = all_wait(h_empty, (h_per++ & 1u) ^ 1u))) break;
+        fence_after();
+        for (uint32_t j = 0; j < lead; ++j) issue_h(s + j, true);
+        s += lead;
+      } else if (l_opens) {
+        // the H products of the next stages run while Lo is drained (at s = 0 both begin)
+        if (h_opens && !(ok = all_wait(h_empty, (h_per++ & 1u) ^ 1u))) break;
+        for (uint32_t j = 0; j < lead && ok; ++j) {
+          if (!(ok = wait_stage(s + j))) break;
+          fence_after();
+          issue_h(s + j, false);
         }
+        if (!ok || !(ok = all_wait(l_empty, (l_per++ & 1u) ^ 1u))) break;
+        fence_after();
+        for (uint32_t j = 0; j < lead; ++j) issue_l(s + j, true);
+        s += lead;
       } else {
-#pragma unroll
-        for (uint32_t g = 0; g < 128 / W; ++g) {
-          uint32_t r[W];
-          ld_(g, r);
-          tmem_wait_ld();
-          f(g, r);
-          fill_(g);
-        }
+        if (!(ok = wait_stage(s))) break;
+        fence_after();
+        issue_h(s, false);
+        issue_l(s, true);
+        ++s;
       }
+    }
+    // every MMA issued above completes before the tensor memory is freed
+    if (elect_one()) umma_commit(done_bar);
+    __syncwarp();
+    mbar_wait(done_bar, 0, p.status, nullptr);
+  } else if (warp == 2) {
+    // ------------------------------- raw copies ---------------------------------
+    Ring r;
+    uint32_t issued = 0;
+    for (uint32_t kb = kb0; kb < kb0 + nst; kb += KBR) {
+      if (!all_wait(r_empty + 8 * r.s, r.ph ^ 1u)) break;
+      if (elect_one()) {
+        const uint32_t full = r_full + 8 * r.s, base = rring + r.s * RAW_STAGE;
+        uint32_t seg;
+        const int32_t kx = k_of(kb, seg);
+        mbar_expect_tx(full, RAW_STAGE);
+#pragma unroll
+        for (uint32_t t = 0; t < 4; ++t)
+          tma_load(base + t * RAW_TILE, &maps.x[seg][t], kx, static_cast<int32_t>(d0), full);
+      }
+      __syncwarp();
+      ++issued;
+      r.next(p.nr);
+    }
+    if (*abort) {
+      for (uint32_t G = issued > p.nr ? issued - p.nr : 0; G < issued; ++G)
+        mbar_wait(r_full + 8 * (G % p.nr), (G / p.nr) & 1u, p.status, nullptr);
+    }
+  } else if (warp == 3) {
+    // a widened stage's full barrier also counts the arrival of its query tiles; a_empty keeps the turn
+    for (uint32_t G = 0; G < nst; ++G) {
+      if (G % KBR == 0 && !all_wait(q_full + 8 * stage_of<NQ>(G / KBR), phase_of<NQ>(G / KBR))) break;
+      if (!all_wait(a_empty + 8 * stage_of<NA>(G), phase_of<NA>(G) ^ 1u)) break;
+      if (lane == 0) mbar_arrive(a_full + 8 * stage_of<NA>(G));
+    }
+  } else if (warp >= ISSUE_WARPS + DW) {
+    // -------------------------------- widening ----------------------------------
+    // the first four warps take the even k-blocks (a raw stage's first), the others the odd ones
+    const uint32_t kr = (warp - ISSUE_WARPS - DW) >> 2, row = 32 * (warp & 3u) + lane, x = (row >> 1) & 3u;
+    const uint32_t lane_base = (32u * (warp & 3u)) << 16;
+    // chunks 2 kr, 2 kr + 1 of the 64-byte swizzled row
+    const uint32_t o0 = ((2 * kr) ^ x) * 16, o1 = ((2 * kr + 1) ^ x) * 16;
+    Ring r;
+    for (uint32_t G = kr; G < nst; G += KBR) {
+      if (!all_wait(r_full + 8 * r.s, r.ph)) break;
+      const uint32_t src = rring + r.s * RAW_STAGE + row * KR, dst = tA + lane_base + stage_of<NA>(G) * A_COLS;
+      uint32_t w[32];
+      auto widen = [&](uint32_t limb) {  // this row's 32 elements of limbs `limb` and `limb` + 1
+        const uint32_t t0 = src + limb * RAW_TILE, t1 = t0 + RAW_TILE;
+        const uint4 v[4] = {lds128(t0 + o0), lds128(t0 + o1), lds128(t1 + o0), lds128(t1 + o1)};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          uint4 c0, c1;
+          widen16(v[e], c0, c1);
+          w[8 * e] = c0.x, w[8 * e + 1] = c0.y, w[8 * e + 2] = c0.z, w[8 * e + 3] = c0.w;
+          w[8 * e + 4] = c1.x, w[8 * e + 5] = c1.y, w[8 * e + 6] = c1.z, w[8 * e + 7] = c1.w;
+        }
+      };
+      widen(0);
+      if (!all_wait(a_empty + 8 * stage_of<NA>(G), phase_of<NA>(G) ^ 1u)) break;
+      fence_after();
+      tmem_st32(dst, w);
+      widen(2);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(r_empty + 8 * r.s);
+      r.next(p.nr);
+      tmem_st32(dst + 32, w);
       tmem_wait_st();
       fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(a_empty + 8 * region);
+      if (lane == 0) mbar_arrive(a_full + 8 * stage_of<NA>(G));
+    }
+  } else {
+    // ----------------------------------- drain ----------------------------------
+    const uint32_t half = (warp - ISSUE_WARPS) >> 2, span = (nw / 16 + 1) / 2 * 16, col0 = half * span;
+    const uint32_t ng = col0 < nw ? ((nw - col0 < span ? nw - col0 : span) / 16) : 0;
+    const uint32_t t0 = tmem + ((32u * (warp & 3u)) << 16) + col0;
+    uint32_t acc[16 * MAXG];  // this row's sums of the warp's columns mod 2^32
+#pragma unroll
+    for (uint32_t k = 0; k < 16 * MAXG; ++k) acc[k] = 0;
+    // one drain: the pair of accumulators at t, 16 columns of each at a time, to f; then the pair is released
+    auto drain = [&](uint32_t full, uint32_t par, uint32_t t, uint32_t empty, auto&& f) {
+      if (!all_wait(full, par)) return false;
+      fence_after();
+#pragma unroll
+      for (uint32_t g = 0; g < MAXG; ++g) {
+        if (g < ng) {
+          uint32_t a[16], b[16];
+          tmem_ld16(t + 16 * g, a);
+          tmem_ld16(t + tn + 16 * g, b);
+          tmem_wait_ld();
+          if (g == ng - 1) {  // the last of this warp's columns is in registers
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty);
+          }
+          f(g, a, b);
+        }
+      }
+      if (ng == 0 && lane == 0) mbar_arrive(empty);
       return true;
     };
+    uint32_t h_per = 0, l_per = 0;
     bool ok = true;
-    {
-      // pass A: u[k] holds U mod 2^16 of columns 2k (low half) and 2k + 1 (high half); bits(M)
-      // is 0 mod 2^16, so the raw bits of a drained S_2 add as they are, S_3's shifted by 8
-      uint32_t u[64];
+    for (uint32_t s = 1; s <= nst && ok; ++s) {
+      if (s % HP == 0 || s == nst)
+        ok = drain(h_full, h_per++ & 1u, t0 + 2 * tn, h_empty, [&](uint32_t g, const uint32_t (&a)[16], const uint32_t (&b)[16]) {
 #pragma unroll
-      for (int k = 0; k < 64; ++k) u[k] = 0;
-      for (uint32_t d = 0; d < kbt / 2 && ok; ++d) {
-        ok = drain(
-            1, done1,
-            [&](uint32_t g, const uint32_t (&r)[32]) {
+          for (int k = 0; k < 8; ++k) {
+            const uint32_t u = add16x2(low16x2<1>(a[2 * k], a[2 * k + 1]), low16x2<256>(b[2 * k], b[2 * k + 1]));
+            acc[16 * g + 2 * k] += u << 16;
+            acc[16 * g + 2 * k + 1] += u & 0xFFFF0000u;
+          }
+        });
+      if (ok && (s % LP == LOFF || s == nst))
+        ok = drain(l_full, l_per++ & 1u, t0, l_empty, [&](uint32_t g, const uint32_t (&a)[16], const uint32_t (&b)[16]) {
 #pragma unroll
-              for (int k = 0; k < 16; ++k) u[16 * g + k] = add16x2(u[16 * g + k], pack_c16(r[2 * k], r[2 * k + 1]));
-            },
-            std::integral_constant<uint32_t, 32>{});
-        if (ok)
-          ok = drain(
-              0, done0,
-              [&](uint32_t g, const uint32_t (&r)[32]) {
+          for (int k = 0; k < 16; ++k)
+            acc[16 * g + k] += static_cast<uint32_t>(__float2int_rn(__uint_as_float(a[k]))) +
+                               (static_cast<uint32_t>(__float2int_rn(__uint_as_float(b[k]))) << 8);
+        });
+    }
+    // ---- epilogue: the sums through the (now idle) query ring, then four rows of a column at a time ----
+    if (!named_sync_or(1, DT, *abort != 0)) {
+      uint32_t* zs = reinterpret_cast<uint32_t*>(smem);  // [tn][TM]
+      const uint32_t row = 32 * (warp & 3u) + lane;
 #pragma unroll
-                for (int k = 0; k < 16; ++k)
-                  u[16 * g + k] = add16x2(u[16 * g + k], pack_lo16(r[2 * k], r[2 * k + 1]));
-              },
-              std::integral_constant<uint32_t, 32>{});
+      for (uint32_t k = 0; k < 16 * MAXG; ++k)
+        if (k < 16 * ng) zs[(col0 + k) * TM + row] = acc[k];
+      if (!SPLIT) {
+        named_sync(1, DT);
+        for (uint32_t it = threadIdx.x - ISSUE_WARPS * 32; it < nw * (TM / 4); it += DT)
+          put_z(q0 + it / (TM / 4), d0 + 4 * (it % (TM / 4)), *reinterpret_cast<const uint4*>(zs + it * 4));
       }
-      // U << 16 goes to z, where the epilogue adds pass B's sums and the zero shares to it
-      if (ok && row < p.x_rows) {
-#pragma unroll
-        for (int k = 0; k < 64; ++k) {
-          const uint32_t c = q0 + 128 * h + 2 * k;
-          if (c < p.n_cols) p.z[static_cast<uint64_t>(c) * p.ldz + row] = u[k] << 16;
-          if (c + 1 < p.n_cols) p.z[static_cast<uint64_t>(c + 1) * p.ldz + row] = u[k] & 0xFFFF0000u;
+    }
+  }
+  if (SPLIT) {
+    // every thread of every CTA passes both cluster barriers, also after a failed wait
+    __syncwarp();
+    cluster_sync();
+    if (warp >= ISSUE_WARPS && warp < ISSUE_WARPS + DW) {
+      bool bad = false;
+      for (uint32_t r = 0; r < n_rank; ++r) bad = bad || ld_cluster32(mapa(smem_addr(&s_abort), r)) != 0;
+      if (!bad)
+        for (uint32_t it = rank * DT + threadIdx.x - ISSUE_WARPS * 32; it < nw * (TM / 4); it += n_rank * DT) {
+          uint4 v = make_uint4(0, 0, 0, 0);
+          for (uint32_t r = 0; r < n_rank; ++r) {
+            const uint4 o = ld_cluster128(mapa(qring + it * 16, r));
+            v = make_uint4(v.x + o.x, v.y + o.y, v.z + o.z, v.w + o.w);
+          }
+          put_z(q0 + it / (TM / 4), d0 + 4 * (it % (TM / 4)), v);
         }
-      }
     }
-    // pass B: 32-bit sums; each S_1 drain adds bits(M) << 8 and each S_0 drain bits(M) once too
-    // often, subtracted up front
-    const uint32_t corr = 0u - (kbt / 4) * (MAGIC << 8) - (kbt / 8) * MAGIC;
-    uint32_t acc[128];
-#pragma unroll
-    for (int k = 0; k < 128; ++k) acc[k] = corr;
-    for (uint32_t j = 0; j < kbt / 2 && ok; ++j) {
-      if ((j & 1u) == 1)
-        ok = drain(
-            1, done1,
-            [&](uint32_t g, const uint32_t (&r)[16]) {
-#pragma unroll
-              for (int k = 0; k < 16; ++k) acc[16 * g + k] += r[k] << 8;
-            },
-            std::integral_constant<uint32_t, 16>{});
-      if (ok && (j & 3u) == 3)
-        ok = drain(
-            0, done0,
-            [&](uint32_t g, const uint32_t (&r)[16]) {
-#pragma unroll
-              for (int k = 0; k < 16; ++k) acc[16 * g + k] += r[k];
-            },
-            std::integral_constant<uint32_t, 16>{});
-    }
-    // ---- epilogue: z = U << 16 + pass B + r_i, r_i = F(seed_own) - F(seed_prev) (App. C) ----
-    // The sums go to shared memory (the Q ring is idle: the last S_0-full followed every MMA,
-    // and every copy was consumed), then each (column, 4-row group) item adds U << 16 (from z)
-    // and the zero shares of its four rows, one Philox block per seed, and writes 16 bytes of z.
-    named_sync(1, DRAIN_THREADS);
-    if (!*abort) {  // uniform: read after the barrier that every drainer reaches
-      uint32_t* zs = reinterpret_cast<uint32_t*>(smem);  // [TN][TM]
-      const uint32_t trow = 32 * q + lane;
-#pragma unroll
-      for (int k = 0; k < 128; ++k) zs[(128 * h + k) * TM + trow] = acc[k];
-      named_sync(1, DRAIN_THREADS);
-      const uint32_t dt = threadIdx.x - DRAIN_WARP0 * 32;
-      const uint32_t grp0 = static_cast<uint32_t>((p.row0 + d0) >> 2);
-      const uint32_t ctr3 = (IPC_D_ZA32 << 24) | p.vec;
-      for (uint32_t it = dt; it < TN * (TM / 4); it += DRAIN_THREADS) {
-        const uint32_t cc = it / (TM / 4), g4 = it % (TM / 4), col = q0 + cc, r0 = d0 + 4 * g4;
-        if (col >= p.n_cols || r0 >= p.x_rows) continue;
-        const uint32_t req = p.col_tags[2 * col], tag = p.col_tags[2 * col + 1];
-        const uint4 fo = philox(grp0 + g4, tag, req, ctr3, p.seed_own);
-        const uint4 fp = philox(grp0 + g4, tag, req, ctr3, p.seed_prev);
-        const uint4 a = *reinterpret_cast<const uint4*>(zs + cc * TM + 4 * g4);
-        uint32_t* dst = p.z + static_cast<uint64_t>(col) * p.ldz + r0;
-        if (r0 + 4 <= p.x_rows) {
-          const uint4 u = *reinterpret_cast<const uint4*>(dst);
-          const uint4 v = make_uint4(a.x + u.x + fo.x - fp.x, a.y + u.y + fo.y - fp.y, a.z + u.z + fo.z - fp.z,
-                                     a.w + u.w + fo.w - fp.w);
-          __stcs(reinterpret_cast<uint4*>(dst), v);  // streamed: z is read by a later kernel, not from L2
-        } else {
-          const uint32_t av[4] = {a.x, a.y, a.z, a.w}, f[4] = {fo.x - fp.x, fo.y - fp.y, fo.z - fp.z, fo.w - fp.w};
-          for (uint32_t e = 0; e < p.x_rows - r0; ++e) dst[e] = av[e] + dst[e] + f[e];
-        }
-      }
-    }
+    __syncwarp();
+    cluster_sync();
   }
   fence_before();
   __syncthreads();
   if (warp == 0) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
   }
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-int launch_tc32(const Maps32& m, const Tc32Params& p, uint32_t n_cols, size_t x_rows, cudaStream_t stream) {
-  static PerDevice attr;
-  IPC_CUDA_TRY(attr.run(
-      [] { return cudaFuncSetAttribute(gemm_tc32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES); }));
-  const dim3 grid((n_cols + TN - 1) / TN, static_cast<unsigned>((x_rows + TM - 1) / TM));
-  gemm_tc32_kernel<<<grid, THREADS, SMEM_BYTES, stream>>>(m, p);
-  IPC_CUDA_TRY(cudaGetLastError());
+uint32_t cdiv(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
+
+// CTAs that run at once in clusters of k, by device (set with the kernels' attributes).
+uint32_t g_at_once[64][MAX_SPLIT + 1];
+
+cudaError_t ready() {
+  const void* k[4] = {reinterpret_cast<const void*>(&gemm_tc32_kernel<2, false>),
+                      reinterpret_cast<const void*>(&gemm_tc32_kernel<2, true>),
+                      reinterpret_cast<const void*>(&gemm_tc32_kernel<3, false>),
+                      reinterpret_cast<const void*>(&gemm_tc32_kernel<3, true>)};
+  cudaError_t e = cudaSuccess;
+  for (const void* f : k)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+  int dev = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  for (uint32_t s = 2; s <= MAX_SPLIT && e == cudaSuccess && dev >= 0 && dev < 64; ++s) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = s;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(s);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_MAX;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, gemm_tc32_kernel<2, true>, &cfg);
+    g_at_once[dev][s] = e == cudaSuccess ? static_cast<uint32_t>(n) * s : 0;
+  }
+  return e;
+}
+
+// Column tiles and parts of K with the shortest estimate, as for the 16-bit kernel: rounds of the chip x
+// (k-blocks of a CTA x cycles of one + a tile's start and end). A k-block takes 10 cycles a column, and at
+// least 650 at small widths (the raw copies and the widening). 496 columns as six tiles of up to 96 take
+// 5.53 ms, as seven of up to 80, which leave room for a third widened stage, 5.44 ms (30,000 rows, sustained).
+void pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t kb_total, uint32_t& n_ct, uint32_t& split) {
+  int dev = 0;
+  const uint32_t* at_once = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_at_once[dev] : nullptr;
+  const double sms = sm_count_current();
+  const uint32_t units = cdiv(n_cols, 16), least = cdiv(units, MAX_TN / 16);
+  double best = 1e300;
+  for (uint32_t t = least; t <= least + 2 && t <= units; ++t) {
+    const double kb_cycles = std::max(650.0, 10.6 * 16 * cdiv(units, t)), ctas = static_cast<double>(t) * row_tiles;
+    for (uint32_t s = 1; s <= MAX_SPLIT && s <= kb_total / KB_UNIT; ++s) {
+      if (s > 1 && (!at_once || at_once[s] == 0)) continue;
+      const double rounds = ctas * s / (s == 1 ? sms : at_once[s]);
+      const double cost = (rounds < 4 ? std::ceil(rounds) : rounds + 0.5) * (kb_cycles * kb_total / s + (s == 1 ? 10000 : 14000));
+      if (cost < best * 0.999) {
+        best = cost;
+        n_ct = t;
+        split = s;
+      }
+    }
+  }
+}
+
+template <uint32_t NA>
+int launch_tc32(const Maps32& m, const Tc32Params& p, uint32_t split, uint32_t smem, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(p.n_ct * p.n_rt * split);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  if (split > 1) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    at[cfg.numAttrs].val.clusterDim.x = split;
+    at[cfg.numAttrs].val.clusterDim.y = at[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
+  cfg.attrs = at;
+  IPC_CUDA_TRY(cudaLaunchKernelEx(&cfg, split > 1 ? gemm_tc32_kernel<NA, true> : gemm_tc32_kernel<NA, false>, m, p));
   return IPC_OK;
 }
 
@@ -632,19 +662,29 @@ int ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], size_t x_rows, c
     set_error("Z_2^32 ring GEMM: too many rows for one launch");
     return IPC_EINVAL;
   }
+  static PerDevice attr;
+  IPC_CUDA_TRY(attr.run(ready));
+  Tc32Params p{};
+  p.n_rt = static_cast<uint32_t>((x_rows + TM - 1) / TM);
+  p.n_ct = 1;
+  uint32_t split = 1;
+  pick_shape(n_cols, p.n_rt, segments * l / KB, p.n_ct, split);
+  p.tn = 16 * cdiv(cdiv(n_cols, 16), p.n_ct);
+  const uint32_t q_stage = 4 * p.tn * 128;
+  p.nr = std::min(MAX_NR, (SMEM_MAX - 1024 - 8 * NUM_BARS - NQ * q_stage) / RAW_STAGE);
+  const uint32_t smem = 1024 + NQ * q_stage + p.nr * RAW_STAGE + 8 * NUM_BARS;
   Maps32 m;
   int rc;
   for (int i = 0; i < 4; ++i) {
-    if ((rc = make_map_f16(&m.b[i], b[i], static_cast<uint64_t>(segments) * l, n_pad, TN)) ||
-        (rc = make_map_i8(&m.a0[i], x[i], l, x_rows, TM)) ||
-        (rc = make_map_i8(&m.a1[i], x[segments == 2 ? 4 + i : i], l, x_rows, TM)))
+    if ((rc = make_map_f16k64(&m.b[i], b[i], static_cast<uint64_t>(segments) * l, n_pad, p.tn)) ||
+        (rc = make_map_raw(&m.x[0][i], x[i], l, x_rows, KR, TM)) ||
+        (rc = make_map_raw(&m.x[1][i], x[segments == 2 ? 4 + i : i], l, x_rows, KR, TM)))
       return rc;
   }
-  Tc32Params p;
   p.n_cols = n_cols;
   p.x_rows = static_cast<uint32_t>(x_rows);
-  p.kb_total = segments * l / KB;
-  p.kb_half = l / KB;
+  p.segs = segments;
+  p.kb_seg = l / KB;
   p.col_tags = col_tags;
   p.seed_own = seed_own;
   p.seed_prev = seed_prev;
@@ -653,7 +693,8 @@ int ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], size_t x_rows, c
   p.ldz = ldz;
   p.row0 = row0;
   p.status = status_ptr();
-  return launch_tc32(m, p, n_cols, x_rows, stream);
+  return p.tn > 80 ? launch_tc32<2>(m, p, split, smem, stream)
+                   : launch_tc32<3>(m, p, split, smem, stream);
 }
 
 int prep_query32(const uint32_t* y, uint64_t y_plane, uint32_t Q, const ipc_geom* g, uint32_t party,
