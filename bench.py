@@ -7,7 +7,7 @@ copy of the bit components. Workload (default): 100,000 database rows x 32 queri
 rotations, 12,800-bit codes, synthetic (seeded), database shares resident on the device.
 
 Prints one JSON line. `value` is comparisons/s of the tcgen05 path (the resident int8 limb
-planes widened to fp16 in shared memory, exact, fp32 accumulators in tensor memory) with the
+planes widened to fp16 on the way into tensor memory, exact, fp32 accumulators in tensor memory) with the
 query shares already on the device, timed with CUDA events on the library's control stream;
 `e2e` is the same through host (pinned) buffers with the copies inside the timed region, timed
 by the host's clock from the first submit to the last fetched result; `int8_mix_path`,
@@ -620,12 +620,12 @@ def run_ours(args, w):
     peak_imad = ipc.ipc_measure_peak(1)
     peak_dp4a = ipc.ipc_measure_peak(2)
     achieved = ops / (t_tc * 1e-3) / 1e12
-    traffic = ncu_traffic("gemm_tc_kernel", os.path.join(ROOT, "paper_2405_04463_gb300", "csrc", "gemm_tc.cu"))
+    traffic = ncu_traffic("gemm_ts_kernel", os.path.join(ROOT, "paper_2405_04463_gb300", "csrc", "gemm_ts.cu"))
     # algorithmic bytes of one launch: the two database components' int8 limb planes (the size
     # of their u16 shares), the fp16 query operand and z
     alg_bytes = 2 * 2 * rows * l + 2 * 2 * n_pad * 2 * l + 2 * N * rows
     roofline = {"bound": "tensor",
-                "kernel": "gemm_tc_kernel (tcgen05.mma kind::f16; int8 database limbs widened to fp16 in shared "
+                "kernel": "gemm_ts_kernel (tcgen05.mma kind::f16; int8 database limbs widened to fp16 into tensor "
                           "memory, fp16 query limbs; exact)",
                 "achieved": achieved, "peak": bf16_burst, "unit": "TFLOP/s",
                 "frac": achieved / bf16_burst if bf16_burst else None, "traffic": traffic,

@@ -772,17 +772,7 @@ int ring_gemm_ts_group(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32
     }
     kb_most = std::max(kb_most, g[i].segments * l / KB);
   }
-  static PerDevice attr;
-  IPC_CUDA_TRY(attr.run([] {
-    cudaError_t e = ready<Cfg64>();
-    if (e == cudaSuccess) e = ready<Cfg96>();
-    if (e == cudaSuccess) e = ready<Cfg128>();
-    if (e == cudaSuccess) e = ready<Cfg160>();
-    if (e == cudaSuccess) e = ready<Cfg192>();
-    if (e == cudaSuccess) e = ready<Cfg208>();
-    for (uint32_t k = 2; k <= MAX_SPLIT && e == cudaSuccess; ++k) e = clusters_at_once(k);
-    return e;
-  }));
+  if (const int rc = ring_gemm_ts_ready()) return rc;
   TsParams p{};
   TsMaps m;
   const uint32_t sms = static_cast<uint32_t>(sm_count_current());
@@ -863,6 +853,21 @@ int ring_gemm_ts_group(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32
 }
 
 }  // namespace
+
+int ring_gemm_ts_ready() {
+  static PerDevice attr;
+  IPC_CUDA_TRY(attr.run([] {
+    cudaError_t e = ready<Cfg64>();
+    if (e == cudaSuccess) e = ready<Cfg96>();
+    if (e == cudaSuccess) e = ready<Cfg128>();
+    if (e == cudaSuccess) e = ready<Cfg160>();
+    if (e == cudaSuccess) e = ready<Cfg192>();
+    if (e == cudaSuccess) e = ready<Cfg208>();
+    for (uint32_t k = 2; k <= MAX_SPLIT && e == cudaSuccess; ++k) e = clusters_at_once(k);
+    return e;
+  }));
+  return IPC_OK;
+}
 
 // The passes of a launch follow one another, so that two passes' query operands are in use at once: as long
 // as those fit the L2 together all passes run in one launch, which fills the chip best (three passes of

@@ -18,6 +18,10 @@ struct RingGemm {
   uint16_t* z;                      // [n_cols][ldz]
 };
 
+// Loads every form of the kernel on this device (once). Loading one may wait for the work on the device, so
+// contexts call this when they are made; without it the first launch does.
+int ring_gemm_ts_ready();
+
 // n_pass ring GEMMs over the same rows and columns in one launch. col_tiles (device, may be null): the
 // column tiles of list_cols columns to compute, n_col_list (device) their count, walked by one CTA per SM.
 int ring_gemm_ts(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,

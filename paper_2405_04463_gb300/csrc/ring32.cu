@@ -640,6 +640,13 @@ int launch_tc32(const Maps32& m, const Tc32Params& p, uint32_t split, uint32_t s
 
 }  // namespace
 
+// As ring_gemm_ts_ready.
+int ring_gemm_tc32_ready() {
+  static PerDevice attr;
+  IPC_CUDA_TRY(attr.run(ready));
+  return IPC_OK;
+}
+
 // segments: 2 for K = 2l over [x[0..3] | x[4..7]] (ABY3 replicated sharing, x[4..7] the
 // previous party's component), 1 for K = l over x[0..3] alone. K must be a multiple of 256.
 int ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], size_t x_rows, const uint16_t* const b[4],
@@ -662,8 +669,7 @@ int ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], size_t x_rows, c
     set_error("Z_2^32 ring GEMM: too many rows for one launch");
     return IPC_EINVAL;
   }
-  static PerDevice attr;
-  IPC_CUDA_TRY(attr.run(ready));
+  if (const int rc = ring_gemm_tc32_ready()) return rc;
   Tc32Params p{};
   p.n_rt = static_cast<uint32_t>((x_rows + TM - 1) / TM);
   p.n_ct = 1;
