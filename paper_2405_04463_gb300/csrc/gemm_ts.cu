@@ -627,6 +627,7 @@ __global__ void __launch_bounds__(F::THREADS, 1)
       named_sync(1, DT);
       for (uint32_t it = threadIdx.x - ISSUE_WARPS * 32; it < nw * (TM / 8); it += DT)
         put_z(p.pass[ps], q0 + it / (TM / 8), d0 + 8 * (it % (TM / 8)), *reinterpret_cast<const uint4*>(zs + it * 8));
+      fence_proxy_async();  // the next item's query copies overwrite zs through the async proxy
       __syncwarp();
       if (lane == 0) mbar_arrive(epi_done);
     }
