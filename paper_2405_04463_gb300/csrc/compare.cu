@@ -17,6 +17,7 @@ namespace {
 using namespace cmp;
 
 constexpr int CT = 64;  // threads per CTA
+constexpr int COMPARE_SMEM = sizeof(uint32_t) * S_WORDS * CT;
 constexpr uint64_t PLAIN_THREADS = 300000;  // about four times what the chip holds at once
 // One thread per part of each (column, OR block) unit, the parts of a unit in consecutive lanes,
 // joined by warp shuffles; the modes are those of part_root.
@@ -188,6 +189,29 @@ __global__ void __launch_bounds__(32 * 31) or_tree_kernel(uint32_t* roots, uint6
   bit_shares[2 * Q + q] = x.c2 & 1u;
 }
 
+}  // namespace
+
+// Loads the comparison phase's kernels on this device (once).
+int compare_ready() {
+  static tc::PerDevice attr;  // a kernel attribute belongs to one device's context
+  IPC_CUDA_TRY(attr.run([] {
+    cudaError_t e = cudaFuncSetAttribute(compare_kernel<MODE_LIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         COMPARE_SMEM);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(compare_kernel<MODE_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, COMPARE_SMEM);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(compare_kernel<MODE_LIFTFREE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               COMPARE_SMEM);
+    if (e == cudaSuccess)
+      e = tc::load_kernels({reinterpret_cast<const void*>(&or_tree_kernel),
+                            reinterpret_cast<const void*>(&or_join_parts_kernel)});
+    return e;
+  }));
+  return IPC_OK;
+}
+
+namespace {
+
 int launch_compare(CmpParams& P, const uint64_t seeds[3], int mode, cudaStream_t st) {
   if (P.p > 5) {  // a part's OR stack holds levels 0..5 - LOG2_SPLIT
     set_error("compare: log2_block_words must be <= 5");
@@ -204,26 +228,14 @@ int launch_compare(CmpParams& P, const uint64_t seeds[3], int mode, cudaStream_t
   while (P.ks < P.p && (units << P.ks) < PLAIN_THREADS) ++P.ks;
   const uint64_t threads = units << P.ks;
   const Seeds sd = make_seeds(seeds);
-  const size_t smem = sizeof(uint32_t) * S_WORDS * CT;
-  static tc::PerDevice attr;  // a kernel attribute belongs to one device's context
-  IPC_CUDA_TRY(attr.run([smem] {
-    cudaError_t e = cudaFuncSetAttribute(compare_kernel<MODE_LIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(compare_kernel<MODE_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(smem));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(compare_kernel<MODE_LIFTFREE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(smem));
-    return e;
-  }));
+  if (const int rc = compare_ready()) return rc;
   const unsigned grid = static_cast<unsigned>((threads + CT - 1) / CT);
   if (mode == MODE_PLAIN)
-    compare_kernel<MODE_PLAIN><<<grid, CT, smem, st>>>(P, sd);
+    compare_kernel<MODE_PLAIN><<<grid, CT, COMPARE_SMEM, st>>>(P, sd);
   else if (mode == MODE_LIFTFREE)
-    compare_kernel<MODE_LIFTFREE><<<grid, CT, smem, st>>>(P, sd);
+    compare_kernel<MODE_LIFTFREE><<<grid, CT, COMPARE_SMEM, st>>>(P, sd);
   else
-    compare_kernel<MODE_LIFT><<<grid, CT, smem, st>>>(P, sd);
+    compare_kernel<MODE_LIFT><<<grid, CT, COMPARE_SMEM, st>>>(P, sd);
   IPC_CUDA_TRY(cudaGetLastError());
   return IPC_OK;
 }

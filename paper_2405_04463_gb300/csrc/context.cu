@@ -72,16 +72,14 @@ void free_slot(Slot& s) {
   s = Slot();
 }
 
+// Allocated once: no buffer is given back here, which would wait for all work on the device, the caller's
+// included.
 int ensure_zbuf(ipc_ctx* c, uint32_t n_pad) {
   if (c->cfg.keep_distances) return IPC_OK;
   if (c->zbuf_cols >= n_pad) return IPC_OK;
-  CTX_TRY(c, cudaDeviceSynchronize());
-  cudaFree(c->zbuf);
-  c->zbuf = nullptr;
   const size_t bytes = 2ull * 2 * 3 * n_pad * static_cast<size_t>(c->cfg.db_chunk_rows) * c->zsz;
   if (cudaMalloc(&c->zbuf, bytes) != cudaSuccess) {
     cudaGetLastError();
-    c->zbuf_cols = 0;
     return fail(c, IPC_ENOMEM, "cannot allocate the dot-product scratch for " + std::to_string(n_pad) + " columns");
   }
   c->zbuf_cols = n_pad;
@@ -159,6 +157,21 @@ int wait_event(ipc_ctx* c, cudaEvent_t ev, int timeout_ms) {
     else
       std::this_thread::sleep_for(std::chrono::microseconds(50));
   }
+}
+
+// Loads the kernels of a context's requests: loading one at its first launch waits for the work on the
+// device, the caller's included, and a submit does not wait.
+int load_request_kernels(const ipc_config& cfg) {
+  const bool tensor = cfg.path == IPC_PATH_TC || cfg.path == IPC_PATH_TCG;
+  status_ptr();  // the status word's first use clears it, on the default stream
+  int rc = prep_query_ready(tensor, cfg.path == IPC_PATH_TCG || cfg.plain_mask);
+  if (rc == IPC_OK) rc = compare_ready();
+  if (rc != IPC_OK) return rc;
+  if (cfg.path == IPC_PATH_I32) return ring_gemm_i32_ready();
+  if (!tensor) return ring_gemm_i8_ready(cfg.path == IPC_PATH_I8MMA ? 0 : 1);
+  if (cfg.fused) return ring_gemm_compare_ready();
+  rc = ring_gemm_ts_ready();
+  return rc == IPC_OK && cfg.lift ? ring_gemm_tc32_ready() : rc;
 }
 
 // Device inputs are produced by the caller's work on c->input_stream; the library's streams
@@ -242,10 +255,7 @@ extern "C" int ipc_create(const ipc_config* cfg, ipc_ctx** out) {
     ipc_destroy(c);
     return cfail(nullptr, e, "stream/event creation");
   }
-  // the GEMMs' kernels are loaded here: loading one may wait for the caller's work on the device, and a
-  // submit must not
-  int rc = c->qsz == 2 ? ring_gemm_ts_ready() : IPC_OK;
-  if (rc == IPC_OK && c->qsz == 2 && c->cfg.lift) rc = ring_gemm_tc32_ready();
+  const int rc = load_request_kernels(c->cfg);
   if (rc != IPC_OK) {
     const std::string why = ipc::thread_last_error();
     ipc_destroy(c);

@@ -67,7 +67,13 @@ int compare_launch_tiles(const uint16_t* const z_code[3], const uint16_t* const 
                          uint32_t tile_cols, cudaStream_t st, const uint32_t* col_rows, bool plain);
 int prep_query_galois_strided(const uint16_t* y, uint64_t y_plane, uint32_t Q, const ipc_geom* g, uint32_t party,
                               uint16_t* b_lo, uint16_t* b_hi, uint32_t n_pad, void* stream);
+// Loading of the kernels that a request launches.
+int prep_query_ready(bool f16, bool galois);
 int ring_gemm_tc32_ready();
+int ring_gemm_compare_ready();
+int ring_gemm_i8_ready(int mode);
+int ring_gemm_i32_ready();
+int compare_ready();
 int ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], size_t x_rows, const uint16_t* const b[4],
                    uint32_t n_cols, uint32_t n_pad, uint32_t l, const uint32_t* col_tags, uint64_t seed_own,
                    uint64_t seed_prev, uint32_t vec, uint32_t* z, size_t ldz, uint64_t row0, cudaStream_t stream);

@@ -140,6 +140,13 @@ __global__ void __launch_bounds__(THREADS) gemm_i32_kernel(const Params p) {
 
 }  // namespace
 
+// Loads the kernel on this device.
+int ring_gemm_i32_ready() {
+  cudaFuncAttributes attr;
+  IPC_CUDA_TRY(cudaFuncGetAttributes(&attr, gemm_i32_kernel));
+  return IPC_OK;
+}
+
 int ring_gemm_i32(const int8_t* const x_lo[2], const int8_t* const x_hi[2], size_t x_rows, const int8_t* b_lo,
                   const int8_t* b_hi, uint32_t n_cols, uint32_t l, const uint32_t* col_tags, uint64_t seed_own,
                   uint64_t seed_prev, uint32_t vec, uint16_t* z, size_t ldz, uint64_t row0, cudaStream_t stream) {

@@ -553,6 +553,13 @@ int ring_gemm_i8_variant(int variant, const int8_t* const x_lo[2], const int8_t*
   }
 }
 
+// Loads the kernel of ring_gemm_i8's mode on this device.
+int ring_gemm_i8_ready(int mode) {
+  IPC_CUDA_TRY(tc::load_kernels({mode == 1 ? reinterpret_cast<const void*>(&gemm_i8_kernel<1, 128, false>)
+                                           : reinterpret_cast<const void*>(&gemm_i8_kernel<0, 128, false>)}));
+  return IPC_OK;
+}
+
 int ring_gemm_i8(int mode, const int8_t* const x_lo[2], const int8_t* const x_hi[2], size_t x_rows, const int8_t* b_lo,
                  const int8_t* b_hi, uint32_t n_cols, uint32_t n_pad, uint32_t l, const uint32_t* col_tags,
                  uint64_t seed_own, uint64_t seed_prev, uint32_t vec, uint16_t* z, size_t ldz, uint64_t row0,

@@ -512,6 +512,15 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 }  // namespace
 
+// Loads the kernel on this device (once).
+int ring_gemm_compare_ready() {
+  static PerDevice attr;
+  IPC_CUDA_TRY(attr.run([] {
+    return cudaFuncSetAttribute(gemm_cmp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<256>::SMEM_BYTES);
+  }));
+  return IPC_OK;
+}
+
 // The fused chunk step: the six ring GEMMs of a chunk (replicated sharing, segments = 2: party i
 // reads components i and i - 1 of each vector; Galois-ring Shamir shares, segments = 1: party i
 // reads its own share) and the comparison phase of every tile, in one persistent launch of one CTA
@@ -565,10 +574,7 @@ int ring_gemm_compare_tc(uint32_t segments, const int8_t* const x_lo[6], const i
   fp.thr_a = thr_a;
   fp.part_roots = part_roots;
   fp.ld_parts = ld_parts;
-  static PerDevice attr;
-  IPC_CUDA_TRY(attr.run([] {
-    return cudaFuncSetAttribute(gemm_cmp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<256>::SMEM_BYTES);
-  }));
+  if ((rc = ring_gemm_compare_ready())) return rc;
   const uint32_t n_tiles = fp.n_ct * n_rt;
   const uint32_t sms = static_cast<uint32_t>(sm_count_current());
   const dim3 grid(n_tiles < sms ? n_tiles : sms);

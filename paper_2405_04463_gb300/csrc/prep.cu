@@ -4,6 +4,7 @@
 #include <string>
 
 #include "common.cuh"
+#include "tcgen05.cuh"  // load_kernels
 
 namespace ipc {
 namespace {
@@ -393,6 +394,15 @@ extern "C" int ipc_split_limbs(const uint16_t* x, size_t count, int8_t* lo, int8
 }
 
 namespace ipc {
+// Loads the query preparations of a context: fp16 or int8 limbs of replicated shares, or those of Galois-ring
+// shares and public masks.
+int prep_query_ready(bool f16, bool galois) {
+  const void* vec = f16 ? reinterpret_cast<const void*>(&prep_query_vec_kernel<uint16_t>)
+                        : reinterpret_cast<const void*>(&prep_query_vec_kernel<int8_t>);
+  IPC_CUDA_TRY(tc::load_kernels({vec, galois ? reinterpret_cast<const void*>(&prep_query_galois_kernel) : vec}));
+  return IPC_OK;
+}
+
 // y_plane: elements between the three components of y (Q * l when they are packed).
 template <typename T>
 int prep_query_strided(const uint16_t* y, uint64_t y_plane, uint32_t Q, const ipc_geom* g, uint32_t party, T* b_lo,

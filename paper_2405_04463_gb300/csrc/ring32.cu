@@ -571,7 +571,7 @@ cudaError_t ready() {
                       reinterpret_cast<const void*>(&gemm_tc32_kernel<2, true>),
                       reinterpret_cast<const void*>(&gemm_tc32_kernel<3, false>),
                       reinterpret_cast<const void*>(&gemm_tc32_kernel<3, true>)};
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = load_kernels({reinterpret_cast<const void*>(&prep_query32_kernel)});
   for (const void* f : k)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
   int dev = 0;

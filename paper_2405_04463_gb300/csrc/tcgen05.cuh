@@ -6,6 +6,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <initializer_list>
 #include <mutex>
 #include <string>
 
@@ -345,6 +346,16 @@ class PerDevice {
   std::mutex mu_;
   uint64_t done_ = 0;
 };
+
+// Loads kernels on the current device. Code is loaded lazily, at a kernel's first launch, and that waits for
+// the work on the device, the caller's own included.
+inline cudaError_t load_kernels(std::initializer_list<const void*> kernels) {
+  cudaError_t e = cudaSuccess;
+  cudaFuncAttributes attr;
+  for (const void* k : kernels)
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k);
+  return e;
+}
 
 // Number of SMs of the current device.
 inline int sm_count_current() {

@@ -21,8 +21,9 @@ def lib():
 
 
 def dev_u64(a):
+    """Packed bits on the device, copied in the current stream's order without waiting for that stream."""
     torch = torch_mod()
-    return torch.from_numpy(np.ascontiguousarray(a).view(np.int64)).cuda()
+    return torch.from_numpy(np.ascontiguousarray(a).view(np.int64)).to("cuda", non_blocking=True)
 
 
 def galois(path) -> bool:
