@@ -108,7 +108,8 @@ struct Server {
   std::map<std::pair<uint32_t, int>, cudaGraphExec_t> graphs;
 
   std::vector<uint8_t> slot_used;
-  std::deque<SReq*> pending;
+  std::deque<SReq*> placed;   // have their slots; the worker has yet to take them up
+  std::deque<SReq*> pending;  // wait for slots, in submission order
   std::vector<SReq*> active;  // worker thread only
   std::map<uint64_t, std::unique_ptr<SReq>> reqs;
   uint32_t cursor = 0;
@@ -129,6 +130,15 @@ int64_t first_fit(const std::vector<uint8_t>& used, uint32_t want) {
     if (run == want) return static_cast<int64_t>(s + 1 - want);
   }
   return -1;
+}
+
+// Takes free slots for a request; false if there is no run of them (under mu).
+bool place(Server& S, SReq* r) {
+  const int64_t s0 = first_fit(S.slot_used, r->Q);
+  if (s0 < 0) return false;
+  for (uint32_t k = 0; k < r->Q; ++k) S.slot_used[s0 + k] = 1;
+  r->slot0 = static_cast<uint32_t>(s0);
+  return true;
 }
 
 // Sorted distinct tiles of width tw covering the column ranges [col0[i], col0[i] + ncols[i]).
@@ -400,22 +410,21 @@ void worker_main(Server* Sp) {
     std::vector<SReq*> admitted;
     {
       std::unique_lock<std::mutex> lk(S.mu);
-      S.cv_work.wait(lk, [&] { return S.stop || !S.pending.empty() || !S.active.empty(); });
-      if (S.pending.empty() && S.active.empty()) break;  // stop requested and nothing left
+      S.cv_work.wait(lk, [&] { return S.stop || !S.placed.empty() || !S.pending.empty() || !S.active.empty(); });
+      if (S.placed.empty() && S.pending.empty() && S.active.empty()) break;  // stop requested and nothing left
+      while (!S.pending.empty() && place(S, S.pending.front())) {
+        S.placed.push_back(S.pending.front());
+        S.pending.pop_front();
+      }
       const double t = now_s() - S.t0;
-      while (!S.pending.empty()) {
-        SReq* r = S.pending.front();
-        const int64_t s0 = first_fit(S.slot_used, r->Q);
-        if (s0 < 0) break;
-        for (uint32_t k = 0; k < r->Q; ++k) S.slot_used[s0 + k] = 1;
-        r->slot0 = static_cast<uint32_t>(s0);
+      for (SReq* r : S.placed) {
         r->state = 1;
         r->t_admit = t;
         r->chunks_left = S.n_chunks;
-        S.pending.pop_front();
         admitted.push_back(r);
         ++S.admitted;
       }
+      S.placed.clear();
     }
     for (SReq* r : admitted) S.active.push_back(r);
     if (S.active.empty()) continue;
@@ -763,7 +772,8 @@ extern "C" int ipc_serve_submit(ipc_ctx* c, const uint16_t* const code[3], const
   {
     std::lock_guard<std::mutex> lock(S->mu);
     r->t_submit = now_s() - S->t0;
-    S->pending.push_back(r.get());
+    // a request that finds its slots free does not count as waiting while the worker wakes up
+    (S->pending.empty() && place(*S, r.get()) ? S->placed : S->pending).push_back(r.get());
     S->reqs[r->id] = std::move(r);
   }
   S->cv_work.notify_one();
@@ -790,7 +800,7 @@ extern "C" int ipc_serve_stats(ipc_ctx* c, ipc_serve_counters* out) {
   out->steps = S->steps;
   out->admitted = S->admitted;
   out->completed = S->completed;
-  out->pending = S->pending.size();
+  out->pending = S->placed.size() + S->pending.size();
   out->comparisons = S->comparisons;
   out->pool_queries = S->slots;
   out->pool_cols = S->pool_pad;

@@ -107,3 +107,25 @@ def test_full_serving_queue_refuses_until_a_request_is_admitted(torch):
         ipc.ipc_serve_stop(ctx)
     finally:
         ipc.ipc_destroy(ctx)
+
+
+def test_a_request_with_free_slots_does_not_fill_the_queue(torch):
+    """One query slot and one waiting request, the loop idle: of two requests submitted at once the first takes the
+    slot, so the second may wait, however late the loop's thread wakes up."""
+    ipc = lib()
+    w = synth.Workload("held3", s=300, Q=1, planted=1, seed=0xFA16)
+    ctx = make_ctx(w, path="tc", max_queries=1)
+    try:
+        load_workload(ctx, w, chunk=300)
+        code, mask = (v.cpu().numpy() for v in query_shares_gpu(w))
+        ipc.ipc_serve_start(ctx, pool_queries=1, max_pending=1, variant=0)
+        for _ in range(400):
+            rids = [ipc.ipc_serve_submit(ctx, list(code), list(mask), 1) for _ in range(2)]
+            for rid in rids:
+                b = np.zeros(1, np.uint8)
+                ipc.fetch_match_bits(ctx, rid, b, 1, 60000)
+                assert b[0] == 1
+        assert ipc.ipc_serve_stats(ctx)["completed"] == 800
+        ipc.ipc_serve_stop(ctx)
+    finally:
+        ipc.ipc_destroy(ctx)
