@@ -68,6 +68,7 @@ constexpr uint32_t MAX_NR = 8;        // raw stages at most
 constexpr uint32_t SMEM_MAX = 231424;  // dynamic shared memory, leaving room for the static words
 constexpr uint32_t A_COLS = 32;       // TMEM columns of a widened k-block: lo 16, hi 16 (two fp16 a column)
 constexpr uint64_t L2_QUERY_BYTES = 112ull << 20;  // query operands that stay in L2 beside the database
+constexpr double LAUNCH_ROUNDS = 32;  // of the chip, of a launch whose passes' query operands don't fit the L2
 constexpr uint32_t MAX_TN = 208;      // 2 x 208 accumulator columns leave three widened k-blocks
 
 struct TsPass {
@@ -870,26 +871,37 @@ int ring_gemm_ts_ready() {
   return IPC_OK;
 }
 
-// The passes of a launch follow one another, so that two passes' query operands are in use at once: as long
+// The passes of a launch follow one another, so that two passes' query operands are in use at once. As long
 // as those fit the L2 together all passes run in one launch, which fills the chip best (three passes of
-// 51 MB, 30,000 x 496: 4.1 ms against 4.6 ms as three launches); else every pass has its own launch, whose
-// tiles start in step and read the query operand at about the same place. A step of 100,000 rows x 992
-// columns (101 MB of query operand a pass) takes 55.4 ms as six launches a chunk and 62.3 ms as one, at a
-// 20 % lower clock: the tiles drift apart and every one reads its query tiles from DRAM.
+// 51 MB, 30,000 x 496: 4.1 ms against 4.6 ms as three launches). Else tiles drift apart over the rounds of a
+// launch (waves of one tile per SM) until every one reads its query tiles from DRAM, while every launch
+// leaves its last round partly empty: up to 32 rounds all six passes go together, or else a vector's three,
+// or else each alone. Replicated sharing, a request sustained, in ms (six launches / two / one):
+//     16,384 rows x   992 columns ( 4.2 rounds a pass)  9.97 /  9.43 /  9.46
+//     16,384      x 1,984         ( 8.4)               19.22 / 18.96 / 19.98
+//     40,000      x   992         (10.3)               23.15 / 22.69 / 23.92
+//     65,536      x   992         (17)                 36.58 / 38.45 / 40.13
+// Galois-ring shares (K half as long) differ by less than 1 % from 8 rounds a pass on, and 2,000 x 1,984
+// takes 1.80 / 1.57 / 1.48 ms.
+uint32_t ring_gemm_ts_passes(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t cols, uint32_t l) {
+  uint64_t bytes = 0;
+  for (uint32_t i = 0; i < n_pass; ++i) bytes = std::max<uint64_t>(bytes, 4ull * g[i].segments * l * cols);
+  const double rounds = static_cast<double>(cdiv(cols, MAX_TN)) * cdiv(static_cast<uint32_t>(x_rows), TM) / sm_count_current();
+  if (2 * bytes <= L2_QUERY_BYTES || n_pass * rounds <= LAUNCH_ROUNDS) return n_pass;
+  return 3 * rounds <= LAUNCH_ROUNDS ? 3 : 1;
+}
+
 int ring_gemm_ts(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,
                  const uint32_t* col_tags, size_t ldz, uint64_t row0, uint32_t list_cols, const uint32_t* col_tiles,
-                 const uint32_t* n_col_list, cudaStream_t stream) {
+                 const uint32_t* n_col_list, uint32_t cols, cudaStream_t stream) {
   if (n_pass == 0 || n_pass > RING_GEMM_PASSES) {
     set_error("tcgen05 ring GEMM: one to six passes");
     return IPC_EINVAL;
   }
-  uint64_t bytes = 0;
-  for (uint32_t i = 0; i < n_pass; ++i) bytes = std::max<uint64_t>(bytes, 4ull * g[i].segments * l * n_cols);
-  const uint32_t groups = 2 * bytes > L2_QUERY_BYTES ? n_pass : 1;
-  for (uint32_t i = 0; i < groups; ++i) {
-    const uint32_t first = n_pass * i / groups, last = n_pass * (i + 1) / groups;
-    const int rc = ring_gemm_ts_group(last - first, g + first, x_rows, n_cols, n_pad, l, col_tags, ldz, row0, list_cols,
-                                      col_tiles, n_col_list, stream);
+  const uint32_t per = ring_gemm_ts_passes(n_pass, g, x_rows, cols, l);
+  for (uint32_t first = 0; first < n_pass; first += per) {
+    const int rc = ring_gemm_ts_group(std::min(per, n_pass - first), g + first, x_rows, n_cols, n_pad, l, col_tags, ldz,
+                                      row0, list_cols, col_tiles, n_col_list, stream);
     if (rc) return rc;
   }
   return IPC_OK;
@@ -901,7 +913,7 @@ int ring_gemm_tc_variant(uint32_t tile_cols, uint32_t segments, const int8_t* co
                          uint64_t seed_prev, uint32_t vec, uint16_t* z, size_t ldz, uint64_t row0,
                          const uint32_t* col_tiles, const uint32_t* n_col_list, cudaStream_t stream) {
   const RingGemm g{{x_lo[0], x_lo[1]}, {x_hi[0], x_hi[1]}, segments, b_lo, b_hi, seed_own, seed_prev, vec, z};
-  return ring_gemm_ts(1, &g, x_rows, n_cols, n_pad, l, col_tags, ldz, row0, tile_cols, col_tiles, n_col_list, stream);
+  return ring_gemm_ts(1, &g, x_rows, n_cols, n_pad, l, col_tags, ldz, row0, tile_cols, col_tiles, n_col_list, n_cols, stream);
 }
 
 int ring_gemm_tc(const int8_t* const x_lo[2], const int8_t* const x_hi[2], size_t x_rows, const uint16_t* b_lo,

@@ -214,7 +214,7 @@ int gemm_all(Server& S, int v, const Chunk& ch, uint32_t n_pass, cudaStream_t st
                                 z_plane(S, vec, i)};
     }
   return ring_gemm_ts(n_pass, g, ch.rows, S.pool_pad, S.pool_pad, c->l, S.tags, c->cfg.db_chunk_rows, ch.row0,
-                      S.variants[v].tile_cols, S.list_dev[v], S.count_dev[v], st);
+                      S.variants[v].tile_cols, S.list_dev[v], S.count_dev[v], S.pool_pad, st);
 }
 
 // A3 of one party and vector over the listed tiles of the pool, for one chunk (int8 paths).
