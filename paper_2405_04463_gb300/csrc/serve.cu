@@ -68,6 +68,7 @@ struct SReq {
   std::vector<uint8_t> shares;   // [3][Q] bit components, once done
   uint32_t slot0 = 0;
   uint32_t chunks_left = 0;
+  bool room = false;  // there were free slots for it and all before it when it was submitted
   int state = 0;  // 0 pending, 1 active, 2 done
   double t_submit = 0, t_admit = -1, t_done = -1;
   struct Server* srv = nullptr;
@@ -108,8 +109,8 @@ struct Server {
   std::map<std::pair<uint32_t, int>, cudaGraphExec_t> graphs;
 
   std::vector<uint8_t> slot_used;
-  std::deque<SReq*> placed;   // have their slots; the worker has yet to take them up
-  std::deque<SReq*> pending;  // wait for slots, in submission order
+  std::deque<SReq*> pending;
+  uint32_t waiting = 0;       // pending requests that found no free slots when they were submitted
   std::vector<SReq*> active;  // worker thread only
   std::map<uint64_t, std::unique_ptr<SReq>> reqs;
   uint32_t cursor = 0;
@@ -132,13 +133,18 @@ int64_t first_fit(const std::vector<uint8_t>& used, uint32_t want) {
   return -1;
 }
 
-// Takes free slots for a request; false if there is no run of them (under mu).
-bool place(Server& S, SReq* r) {
-  const int64_t s0 = first_fit(S.slot_used, r->Q);
-  if (s0 < 0) return false;
-  for (uint32_t k = 0; k < r->Q; ++k) S.slot_used[s0 + k] = 1;
-  r->slot0 = static_cast<uint32_t>(s0);
-  return true;
+// Whether the worker would admit a request of Q queries behind the pending ones at once (under mu).
+bool has_room(const Server& S, uint32_t Q) {
+  if (S.waiting) return false;
+  std::vector<uint8_t> used = S.slot_used;
+  auto take = [&used](uint32_t n) {
+    const int64_t s0 = first_fit(used, n);
+    if (s0 >= 0) std::fill_n(used.begin() + s0, n, uint8_t(1));
+    return s0 >= 0;
+  };
+  for (const SReq* r : S.pending)
+    if (!take(r->Q)) return false;
+  return take(Q);
 }
 
 // Sorted distinct tiles of width tw covering the column ranges [col0[i], col0[i] + ncols[i]).
@@ -410,21 +416,23 @@ void worker_main(Server* Sp) {
     std::vector<SReq*> admitted;
     {
       std::unique_lock<std::mutex> lk(S.mu);
-      S.cv_work.wait(lk, [&] { return S.stop || !S.placed.empty() || !S.pending.empty() || !S.active.empty(); });
-      if (S.placed.empty() && S.pending.empty() && S.active.empty()) break;  // stop requested and nothing left
-      while (!S.pending.empty() && place(S, S.pending.front())) {
-        S.placed.push_back(S.pending.front());
-        S.pending.pop_front();
-      }
+      S.cv_work.wait(lk, [&] { return S.stop || !S.pending.empty() || !S.active.empty(); });
+      if (S.pending.empty() && S.active.empty()) break;  // stop requested and nothing left
       const double t = now_s() - S.t0;
-      for (SReq* r : S.placed) {
+      while (!S.pending.empty()) {
+        SReq* r = S.pending.front();
+        const int64_t s0 = first_fit(S.slot_used, r->Q);
+        if (s0 < 0) break;
+        for (uint32_t k = 0; k < r->Q; ++k) S.slot_used[s0 + k] = 1;
+        r->slot0 = static_cast<uint32_t>(s0);
         r->state = 1;
         r->t_admit = t;
         r->chunks_left = S.n_chunks;
+        S.pending.pop_front();
+        if (!r->room) --S.waiting;
         admitted.push_back(r);
         ++S.admitted;
       }
-      S.placed.clear();
     }
     for (SReq* r : admitted) S.active.push_back(r);
     if (S.active.empty()) continue;
@@ -748,7 +756,8 @@ extern "C" int ipc_serve_submit(ipc_ctx* c, const uint16_t* const code[3], const
     std::lock_guard<std::mutex> lock(S->mu);
     if (!S->worker_err.empty()) return ctx_fail(c, IPC_ECUDA, "serving loop stopped: " + S->worker_err);
     if (S->stop) return ctx_fail(c, IPC_EINVAL, "ipc_serve_submit: the loop is stopping");
-    if (S->pending.size() >= max_pending) return ctx_fail(c, IPC_EAGAIN, "ipc_serve_submit: pending queue full");
+    // a request that finds its slots free does not fill the queue while the worker wakes up
+    if (S->waiting >= max_pending) return ctx_fail(c, IPC_EAGAIN, "ipc_serve_submit: pending queue full");
   }
   auto r = std::make_unique<SReq>();
   r->Q = static_cast<uint32_t>(n_queries);
@@ -772,8 +781,9 @@ extern "C" int ipc_serve_submit(ipc_ctx* c, const uint16_t* const code[3], const
   {
     std::lock_guard<std::mutex> lock(S->mu);
     r->t_submit = now_s() - S->t0;
-    // a request that finds its slots free does not count as waiting while the worker wakes up
-    (S->pending.empty() && place(*S, r.get()) ? S->placed : S->pending).push_back(r.get());
+    r->room = has_room(*S, r->Q);
+    if (!r->room) ++S->waiting;
+    S->pending.push_back(r.get());
     S->reqs[r->id] = std::move(r);
   }
   S->cv_work.notify_one();
@@ -800,7 +810,7 @@ extern "C" int ipc_serve_stats(ipc_ctx* c, ipc_serve_counters* out) {
   out->steps = S->steps;
   out->admitted = S->admitted;
   out->completed = S->completed;
-  out->pending = S->placed.size() + S->pending.size();
+  out->pending = S->pending.size();
   out->comparisons = S->comparisons;
   out->pool_queries = S->slots;
   out->pool_cols = S->pool_pad;
