@@ -610,7 +610,7 @@ extern "C" int submit_queries(ipc_ctx* c, const uint16_t* const code[3], const u
                                  reinterpret_cast<uint16_t*>(zo)};
         }
       if (n_pass > 0)
-        SUB_RC(ring_gemm_ts(n_pass, g, ch.rows, N, n_pad, l, sl.tags, ldz, ch.row0, 0, nullptr, nullptr, N, c->sp[0]));
+        SUB_RC(ring_gemm_ts(n_pass, g, ch.rows, N, n_pad, l, sl.tags, ldz, ch.row0, c->sp[0]));
       for (int i = 0; i < (c->cfg.lift ? 3 : 1); ++i) {
         SUB_TRY(cudaEventRecord(c->ev_gemm[i][set], c->sp[i]));
         SUB_TRY(cudaStreamWaitEvent(c->sc, c->ev_gemm[i][set], 0));

@@ -883,22 +883,20 @@ int ring_gemm_ts_ready() {
 //     65,536      x   992         (17)                 36.58 / 38.45 / 40.13
 // Galois-ring shares (K half as long) differ by less than 1 % from 8 rounds a pass on, and 2,000 x 1,984
 // takes 1.80 / 1.57 / 1.48 ms.
-uint32_t ring_gemm_ts_passes(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t cols, uint32_t l) {
-  uint64_t bytes = 0;
-  for (uint32_t i = 0; i < n_pass; ++i) bytes = std::max<uint64_t>(bytes, 4ull * g[i].segments * l * cols);
+uint32_t ring_gemm_ts_passes(uint32_t n_pass, uint32_t segments, size_t x_rows, uint32_t cols, uint32_t l) {
+  const uint64_t bytes = 4ull * segments * l * cols;
   const double rounds = static_cast<double>(cdiv(cols, MAX_TN)) * cdiv(static_cast<uint32_t>(x_rows), TM) / sm_count_current();
   if (2 * bytes <= L2_QUERY_BYTES || n_pass * rounds <= LAUNCH_ROUNDS) return n_pass;
   return 3 * rounds <= LAUNCH_ROUNDS ? 3 : 1;
 }
 
-int ring_gemm_ts(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,
-                 const uint32_t* col_tags, size_t ldz, uint64_t row0, uint32_t list_cols, const uint32_t* col_tiles,
-                 const uint32_t* n_col_list, uint32_t cols, cudaStream_t stream) {
-  if (n_pass == 0 || n_pass > RING_GEMM_PASSES) {
+int ring_gemm_ts_by(uint32_t per, uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad,
+                    uint32_t l, const uint32_t* col_tags, size_t ldz, uint64_t row0, uint32_t list_cols,
+                    const uint32_t* col_tiles, const uint32_t* n_col_list, cudaStream_t stream) {
+  if (n_pass == 0 || n_pass > RING_GEMM_PASSES || per == 0) {
     set_error("tcgen05 ring GEMM: one to six passes");
     return IPC_EINVAL;
   }
-  const uint32_t per = ring_gemm_ts_passes(n_pass, g, x_rows, cols, l);
   for (uint32_t first = 0; first < n_pass; first += per) {
     const int rc = ring_gemm_ts_group(std::min(per, n_pass - first), g + first, x_rows, n_cols, n_pad, l, col_tags, ldz,
                                       row0, list_cols, col_tiles, n_col_list, stream);
@@ -907,13 +905,21 @@ int ring_gemm_ts(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_c
   return IPC_OK;
 }
 
+int ring_gemm_ts(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,
+                 const uint32_t* col_tags, size_t ldz, uint64_t row0, cudaStream_t stream) {
+  uint32_t segments = 0;
+  for (uint32_t i = 0; i < n_pass && i < RING_GEMM_PASSES; ++i) segments = std::max(segments, g[i].segments);
+  return ring_gemm_ts_by(ring_gemm_ts_passes(n_pass, segments, x_rows, n_cols, l), n_pass, g, x_rows, n_cols, n_pad, l,
+                         col_tags, ldz, row0, 0, nullptr, nullptr, stream);
+}
+
 int ring_gemm_tc_variant(uint32_t tile_cols, uint32_t segments, const int8_t* const x_lo[2],
                          const int8_t* const x_hi[2], size_t x_rows, const uint16_t* b_lo, const uint16_t* b_hi,
                          uint32_t n_cols, uint32_t n_pad, uint32_t l, const uint32_t* col_tags, uint64_t seed_own,
                          uint64_t seed_prev, uint32_t vec, uint16_t* z, size_t ldz, uint64_t row0,
                          const uint32_t* col_tiles, const uint32_t* n_col_list, cudaStream_t stream) {
   const RingGemm g{{x_lo[0], x_lo[1]}, {x_hi[0], x_hi[1]}, segments, b_lo, b_hi, seed_own, seed_prev, vec, z};
-  return ring_gemm_ts(1, &g, x_rows, n_cols, n_pad, l, col_tags, ldz, row0, tile_cols, col_tiles, n_col_list, n_cols, stream);
+  return ring_gemm_ts_by(1, 1, &g, x_rows, n_cols, n_pad, l, col_tags, ldz, row0, tile_cols, col_tiles, n_col_list, stream);
 }
 
 int ring_gemm_tc(const int8_t* const x_lo[2], const int8_t* const x_hi[2], size_t x_rows, const uint16_t* b_lo,

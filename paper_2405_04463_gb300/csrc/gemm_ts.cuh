@@ -22,15 +22,17 @@ struct RingGemm {
 // contexts call this when they are made; without it the first launch does.
 int ring_gemm_ts_ready();
 
-// n_pass ring GEMMs over the same rows and columns, in as few launches as pay. col_tiles (device, may be
-// null): the column tiles of list_cols columns to compute, n_col_list (device) their count, walked by one CTA
-// per SM. cols: the columns to compute (n_cols, or about as many as the list holds); it decides how many
-// passes a launch takes, nothing else.
+// n_pass ring GEMMs over the same rows and columns, in as few launches as pay.
 int ring_gemm_ts(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,
-                 const uint32_t* col_tags, size_t ldz, uint64_t row0, uint32_t list_cols, const uint32_t* col_tiles,
-                 const uint32_t* n_col_list, uint32_t cols, cudaStream_t stream);
+                 const uint32_t* col_tags, size_t ldz, uint64_t row0, cudaStream_t stream);
 
-// Passes of a launch of that call: n_pass, 3 or 1.
-uint32_t ring_gemm_ts_passes(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t cols, uint32_t l);
+// The passes of a launch that pay for `cols` columns and K of `segments` (the longest pass's): n_pass, 3 or 1.
+uint32_t ring_gemm_ts_passes(uint32_t n_pass, uint32_t segments, size_t x_rows, uint32_t cols, uint32_t l);
+
+// The same with `per` passes in a launch. col_tiles (device, may be null): the column tiles of list_cols
+// columns to compute, n_col_list (device) their count, walked by one CTA per SM.
+int ring_gemm_ts_by(uint32_t per, uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad,
+                    uint32_t l, const uint32_t* col_tags, size_t ldz, uint64_t row0, uint32_t list_cols,
+                    const uint32_t* col_tiles, const uint32_t* n_col_list, cudaStream_t stream);
 
 }  // namespace ipc

@@ -165,7 +165,7 @@ int batch_part(ipc_ctx* c, const uint16_t* const code[3], const uint16_t* const 
       }
     }
   }
-  if (tensor) P_RC(ring_gemm_ts(6, gemms, P, N, n_pad, l, bb.tags, ldz, 0, 0, nullptr, nullptr, N, st));
+  if (tensor) P_RC(ring_gemm_ts(6, gemms, P, N, n_pad, l, bb.tags, ldz, 0, st));
   // A4-A8 with the rows of later persons as public zeros, then the rest of the OR tree
   const uint16_t* zcc[3] = {zc[0], zc[1], zc[2]};
   const uint16_t* zmc[3] = {zm[0], zm[1], zm[2]};

@@ -4,7 +4,7 @@
 // slot, columns q*R + rho as in a stand-alone request). One serving step runs one resident
 // database chunk for every active column: the six share-domain GEMMs (A3; one launch on the tcgen05
 // paths, three party streams on the int8 ones) and the comparison phase (A4-A8 with the in-block OR) over the column tiles that hold active
-// columns, replayed from a CUDA graph keyed by (chunk, GEMM tile variant); the tile list lives
+// columns, replayed from a CUDA graph keyed by (chunk, GEMM tile variant, passes of a launch); the tile list lives
 // in device memory and is rewritten before each replay, so one graph serves every mix of
 // requests. A request admitted while the loop is at chunk c visits chunks c, c+1, ... and
 // after the last one its OR tree is finished (A8) and its bit components copied out; its slots
@@ -21,6 +21,7 @@
 #include <fstream>
 #include <memory>
 #include <sstream>
+#include <tuple>
 
 #include "context.cuh"
 
@@ -106,7 +107,7 @@ struct Server {
   std::vector<uint32_t*> count_dev;  // per variant: 1 word
   uint32_t* list_host[2] = {nullptr, nullptr};  // pinned staging, one per in-flight step
   cudaEvent_t ev_fork = nullptr, ev_join[3] = {}, ev_step[2] = {};
-  std::map<std::pair<uint32_t, int>, cudaGraphExec_t> graphs;
+  std::map<std::tuple<uint32_t, int, uint32_t>, cudaGraphExec_t> graphs;  // by chunk, variant, passes of a launch
 
   std::vector<uint8_t> slot_used;
   std::deque<SReq*> pending;
@@ -197,10 +198,18 @@ uint16_t* z_plane(const Server& S, int vec, int party) {
 
 bool tensor_path(const Server& S) { return S.c->cfg.path == IPC_PATH_TC || S.c->cfg.path == IPC_PATH_TCG; }
 
-// A3 of every party and vector over the listed tiles of the pool, for one chunk (tcgen05 paths):
-// replicated sharing: [own | previous] components, K = 2l; Galois-ring Shamir: own share, K = l.
-// n_pass: the first passes only (one, when the autotuner times a variant).
-int gemm_all(Server& S, int v, const Chunk& ch, uint32_t n_pass, cudaStream_t st) {
+// Passes of one launch over n_tiles listed tiles of variant v: by the step's columns, not the pool's. 0 on
+// the int8 paths, whose GEMMs are launched one by one.
+uint32_t launch_passes(const Server& S, int v, const Chunk& ch, size_t n_tiles) {
+  if (!tensor_path(S)) return 0;
+  return ring_gemm_ts_passes(RING_GEMM_PASSES, S.c->cfg.path == IPC_PATH_TCG ? 1 : 2, ch.rows,
+                             static_cast<uint32_t>(n_tiles) * S.variants[v].tile_cols, S.c->l);
+}
+
+// A3 of every party and vector over the listed tiles of the pool, for one chunk (tcgen05 paths), `per` of the
+// six in a launch: replicated sharing: [own | previous] components, K = 2l; Galois-ring Shamir: own share,
+// K = l. n_pass: the first ones only (a launch, when the autotuner times a variant).
+int gemm_all(Server& S, int v, const Chunk& ch, uint32_t n_pass, uint32_t per, cudaStream_t st) {
   ipc_ctx* c = S.c;
   const bool gal = c->cfg.path == IPC_PATH_TCG;
   auto p16 = [](const uint8_t* p) { return reinterpret_cast<const uint16_t*>(p); };
@@ -219,8 +228,8 @@ int gemm_all(Server& S, int v, const Chunk& ch, uint32_t n_pass, cudaStream_t st
                                 static_cast<uint32_t>(vec),
                                 z_plane(S, vec, i)};
     }
-  return ring_gemm_ts(n_pass, g, ch.rows, S.pool_pad, S.pool_pad, c->l, S.tags, c->cfg.db_chunk_rows, ch.row0,
-                      S.variants[v].tile_cols, S.list_dev[v], S.count_dev[v], S.pool_pad, st);
+  return ring_gemm_ts_by(per, n_pass, g, ch.rows, S.pool_pad, S.pool_pad, c->l, S.tags, c->cfg.db_chunk_rows, ch.row0,
+                         S.variants[v].tile_cols, S.list_dev[v], S.count_dev[v], st);
 }
 
 // A3 of one party and vector over the listed tiles of the pool, for one chunk (int8 paths).
@@ -246,8 +255,8 @@ int compare(Server& S, int v, const Chunk& ch, cudaStream_t st) {
 
 // The graph of one step: the GEMMs (int8 paths: fork the party streams off the control stream, two
 // GEMMs per party, join), then the comparison phase on the control stream.
-int step_graph(Server& S, uint32_t chunk, int v, cudaGraphExec_t* out) {
-  auto it = S.graphs.find({chunk, v});
+int step_graph(Server& S, uint32_t chunk, int v, uint32_t per, cudaGraphExec_t* out) {
+  auto it = S.graphs.find({chunk, v, per});
   if (it != S.graphs.end()) {
     *out = it->second;
     return IPC_OK;
@@ -260,7 +269,7 @@ int step_graph(Server& S, uint32_t chunk, int v, cudaGraphExec_t* out) {
   const bool joint = tensor_path(S);
   cudaError_t e = cudaSuccess;
   if (joint)
-    rc = gemm_all(S, v, ch, RING_GEMM_PASSES, c->sc);
+    rc = gemm_all(S, v, ch, RING_GEMM_PASSES, per, c->sc);
   else
     e = cudaEventRecord(S.ev_fork, c->sc);
   for (int i = 0; !joint && i < 3 && e == cudaSuccess && rc == IPC_OK; ++i) {
@@ -285,7 +294,7 @@ int step_graph(Server& S, uint32_t chunk, int v, cudaGraphExec_t* out) {
   const cudaError_t ei = cudaGraphInstantiate(&exec, g, 0);
   cudaGraphDestroy(g);
   if (ei != cudaSuccess) return ctx_cfail(c, ei, "cudaGraphInstantiate");
-  S.graphs[{chunk, v}] = exec;
+  S.graphs[{chunk, v, per}] = exec;
   *out = exec;
   return IPC_OK;
 }
@@ -381,10 +390,10 @@ int run_step(Server& S, uint64_t step, const std::vector<SReq*>& admitted) {
                          static_cast<uint32_t>(tiles.size())));
   SRV_RC(upload_list(S, v, tiles, step));
   cudaGraphExec_t exec = nullptr;
-  SRV_RC(step_graph(S, S.cursor, v, &exec));
+  const Chunk& ch = c->chunks[S.cursor];
+  SRV_RC(step_graph(S, S.cursor, v, launch_passes(S, v, ch, tiles.size()), &exec));
   SRV_TRY(cudaGraphLaunch(exec, c->sc));
   SRV_TRY(cudaEventRecord(S.ev_step[step & 1], c->sc));
-  const Chunk& ch = c->chunks[S.cursor];
   std::vector<SReq*> still;
   std::vector<SReq*> done;
   for (SReq* r : S.active) {
@@ -450,7 +459,8 @@ void worker_main(Server* Sp) {
 
 // ---------------------------------------------------------------------------------------------
 // Autotuner: per bucket of active columns, the GEMM variant with the shortest launch over the
-// first resident chunk, the listed tiles covering that many columns.
+// first resident chunk, of as many passes as a step launches together, the listed tiles covering
+// that many columns.
 // The table is cached as JSON keyed by device, geometry, chunk rows, path and pool width.
 // ---------------------------------------------------------------------------------------------
 
@@ -519,16 +529,18 @@ int autotune(Server& S) {
       for (uint32_t k = 0; k < tiles.size(); ++k) tiles[k] = k;
       SRV_RC(upload_list(S, v, tiles, 0));
       SRV_TRY(cudaStreamSynchronize(c->sc));
-      // one party and vector, warmed up (which also sets the kernel attributes before any capture)
-      auto once = [&] { return joint ? gemm_all(S, v, ch, 1, c->sc) : gemm(S, v, ch, 0, 0, c->sc); };
-      SRV_RC(once());
+      // a pass as warm-up (which also sets the kernel attributes before any capture), then the passes that
+      // such a step launches together, two launches where it is one
+      const uint32_t per = joint ? launch_passes(S, v, ch, tiles.size()) : 1, reps = per > 1 ? 1 : 2;
+      auto launch = [&](uint32_t n) { return joint ? gemm_all(S, v, ch, n, n, c->sc) : gemm(S, v, ch, 0, 0, c->sc); };
+      SRV_RC(launch(1));
       SRV_TRY(cudaEventRecord(e0, c->sc));
-      for (int rep = 0; rep < 2; ++rep) SRV_RC(once());
+      for (uint32_t rep = 0; rep < reps; ++rep) SRV_RC(launch(per));
       SRV_TRY(cudaEventRecord(e1, c->sc));
       SRV_TRY(cudaEventSynchronize(e1));
       float t = 0;
       SRV_TRY(cudaEventElapsedTime(&t, e0, e1));
-      t /= 2;
+      t /= static_cast<float>(reps * per);  // a pass
       ms << (ms.tellp() > 0 ? ", " : "") << "\"" << S.variants[v].name << "\": " << t;
       if (t < best) {
         best = t;
@@ -721,7 +733,7 @@ extern "C" int ipc_serve_start(ipc_ctx* c, const ipc_serve_config* cfg) {
       rc = autotune(S);
     } else {
       // warm-up launch of the chosen variant (kernel attributes are set outside any capture)
-      rc = tc ? gemm_all(S, cfg->variant, c->chunks[0], 1, c->sc) : gemm(S, cfg->variant, c->chunks[0], 0, 0, c->sc);
+      rc = tc ? gemm_all(S, cfg->variant, c->chunks[0], 1, 1, c->sc) : gemm(S, cfg->variant, c->chunks[0], 0, 0, c->sc);
     }
   }
   if (rc == IPC_OK) {

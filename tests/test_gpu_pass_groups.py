@@ -44,3 +44,41 @@ def test_shares_do_not_depend_on_the_launches(torch, path, plain, rows, Q):
     assert rid == rid2 and (big == small).all()
     bits = big[0] ^ big[1] ^ big[2]
     assert np.nonzero(bits)[0].tolist() == sorted(w.planted_set())
+
+
+@pytest.mark.parametrize("path,rows,pool", [("tc", 4096, 40), ("tc", 40000, 40), ("tcg", 40000, 60)])
+def test_serving_steps_of_every_width(torch, path, rows, pool):
+    """A wide pool with few and with many columns in use: steps of one launch and of several, whichever of them a
+    request shares, give the shares of the same queries submitted alone in small chunks."""
+    ipc = lib()
+    gal = path == "tcg"
+    sizes = [1, 24, 2, pool - 24]
+    w = synth.Workload("steps", s=rows, Q=sum(sizes), planted=4, seed=0x57E9 + rows)
+    qc, qm = w.query_bits()
+    code, mask = query_shares_gpu(w, qc, qm, galois_shares=gal)
+    cuts = np.cumsum([0] + sizes)
+    runs = {}
+    for served in (True, False):
+        ctx = make_ctx(w, path=path, chunk_rows=0 if served else 4096, max_queries=max(sizes))
+        try:
+            load_workload(ctx, w, galois_shares=gal)
+            if served:
+                ipc.ipc_serve_start(ctx, pool_queries=pool)
+            ids = []
+            for a, b in zip(cuts, cuts[1:]):
+                part = [[v[j, a:b].contiguous() for j in range(3)] for v in (code, mask)]
+                if served:
+                    ids.append(ipc.ipc_serve_submit(ctx, *[[t.cpu().numpy() for t in v] for v in part], b - a))
+                else:
+                    ids.append(ipc.submit_queries(ctx, *part, b - a, 1))
+            runs[served] = ids, []
+            for rid, n in zip(ids, sizes):
+                sh = np.zeros((3, n), np.uint8)
+                ipc.fetch_bit_shares(ctx, rid, sh, n, 60000)
+                runs[served][1].append(sh)
+        finally:
+            ipc.ipc_destroy(ctx)
+    assert runs[True][0] == runs[False][0]
+    got, want = (np.concatenate(runs[k][1], 1) for k in (True, False))
+    assert (got == want).all()
+    assert np.nonzero(got[0] ^ got[1] ^ got[2])[0].tolist() == sorted(w.planted_set())
