@@ -492,6 +492,7 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
         const uint32_t n = q0 + dt;
         if (n < p.n_cols) fused_part_compare(p, fp, n, d0 / TM, reinterpret_cast<uint32_t*>(smem), dt);
       }
+      fence_proxy_async();  // the next item's query copies overwrite zs and the scratch through the async proxy
       __syncwarp();
       if (lane == 0) mbar_arrive(epi_done);  // this warp is done with the Q ring
     }
