@@ -33,17 +33,20 @@ __global__ void encode_plain_mask_kernel(const uint64_t* __restrict__ mask_bits,
   *reinterpret_cast<uint4*>(out + static_cast<uint64_t>(r) * l + b0) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// A0: E consecutive bits of a row per thread (blocks_per_row blocks a row), one Philox block per vector and
-// four bits. Bound by the shares it writes; with E = 8 every store has 16 bytes. 8,192 rows of 12,800 bits
-// (1.26 GB): 247 us with E = 4 and a 64-bit division a thread, 201 us so.
+// A0: E consecutive bits of a row per thread, one Philox block per vector and four bits. A block has span
+// threads of each of rows_per_block rows, blocks_per_row blocks a row: a long row takes several blocks, short
+// ones share one. Bound by the shares it writes; with E = 8 every store has 16 bytes. 8,192 rows of 12,800 bits
+// (1.26 GB): 240 us with E = 4 and a 64-bit division a thread, 193 us so; 2^20 rows of 128 bits (1.64 GB):
+// 306 us, 531 us with a block a row, 246 us so.
 template <int E>
 __global__ void encode_share_kernel(const uint64_t* __restrict__ code_bits, const uint64_t* __restrict__ mask_bits,
                                     uint32_t n, uint32_t l, const __grid_constant__ PhiloxKey key, uint32_t side,
-                                    uint32_t idx0, uint32_t blocks_per_row, uint16_t* __restrict__ code_sh,
-                                    uint16_t* __restrict__ mask_sh) {
+                                    uint32_t idx0, uint32_t span, uint32_t rows_per_block, uint32_t blocks_per_row,
+                                    uint16_t* __restrict__ code_sh, uint16_t* __restrict__ mask_sh) {
   static_assert(E == 4 || E == 8, "one or two Philox blocks");
-  const uint32_t r = blockIdx.x / blocks_per_row, t = (blockIdx.x % blocks_per_row) * blockDim.x + threadIdx.x;
-  if (t >= l / E) return;
+  const uint32_t rb = threadIdx.x / span, t = (blockIdx.x % blocks_per_row) * span + (threadIdx.x - rb * span);
+  const uint32_t r = blockIdx.x / blocks_per_row * rows_per_block + rb;
+  if (rb >= rows_per_block || r >= n || t >= l / E) return;
   const uint32_t nw = (l + 63) >> 6, b0 = t * E;
   const uint32_t cw = static_cast<uint32_t>(code_bits[static_cast<uint64_t>(r) * nw + (b0 >> 6)] >> (b0 & 63));
   const uint32_t mw = static_cast<uint32_t>(mask_bits[static_cast<uint64_t>(r) * nw + (b0 >> 6)] >> (b0 & 63));
@@ -352,15 +355,16 @@ extern "C" int ipc_encode_share(const uint64_t* code_bits, const uint64_t* mask_
   if (n == 0) return IPC_OK;
   // 16-byte stores where every row of every component starts on 16 bytes, else 8-byte ones
   const bool wide = l % 8 == 0 && ((reinterpret_cast<uintptr_t>(code_sh) | reinterpret_cast<uintptr_t>(mask_sh)) & 15) == 0;
-  const uint32_t groups = l / (wide ? 8 : 4), bs = groups < 256 ? (groups + 31) / 32 * 32 : 256;
-  const uint32_t per_row = (groups + bs - 1) / bs;
-  if (static_cast<uint64_t>(n) * per_row > 0x7FFFFFFFu) {
+  const uint32_t groups = l / (wide ? 8 : 4), span = groups < 256 ? groups : 256, rows_per_block = 256 / span;
+  const uint32_t bs = (span * rows_per_block + 31) / 32 * 32, per_row = (groups + span - 1) / span;
+  const uint64_t blocks = (static_cast<uint64_t>(n) + rows_per_block - 1) / rows_per_block * per_row;
+  if (blocks > 0x7FFFFFFFu) {
     set_error("ipc_encode_share: too many rows in one call");
     return IPC_EINVAL;
   }
   const PhiloxKey key = philox_key(client_seed);
-  (wide ? encode_share_kernel<8> : encode_share_kernel<4>)<<<n * per_row, bs, 0, as_stream(stream)>>>(
-      code_bits, mask_bits, n, l, key, side, idx0, per_row, code_sh, mask_sh);
+  (wide ? encode_share_kernel<8> : encode_share_kernel<4>)<<<static_cast<unsigned>(blocks), bs, 0, as_stream(stream)>>>(
+      code_bits, mask_bits, n, l, key, side, idx0, span, rows_per_block, per_row, code_sh, mask_sh);
   IPC_CUDA_TRY(cudaGetLastError());
   return IPC_OK;
 }
