@@ -469,7 +469,8 @@ std::string tune_key(const Server& S) {
   cudaGetDeviceProperties(&prop, S.c->cfg.device);
   std::ostringstream k;
   k << prop.name << "|sm" << prop.multiProcessorCount << "|l" << S.c->l << "|rows" << S.c->cfg.db_chunk_rows << "|path"
-    << S.c->cfg.path << "|pool" << S.pool_pad << "|v" << S.n_variants;
+    << S.c->cfg.path << "|pool" << S.pool_pad;
+  if (tensor_path(S)) k << "|v" << S.n_variants;  // their variants were two once, of another kernel
   return k.str();
 }
 
