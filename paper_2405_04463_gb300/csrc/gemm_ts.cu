@@ -120,9 +120,10 @@ struct Sched<4> {
 // (N = 2 tn) and its D [L | C]; two such accumulator pairs take turns, so no drain is waited for. At
 // 32 columns the MMA warp needs 40-50 cycles to issue an MMA of 16, and this saves one in three:
 // 100,000 rows x 62 columns 0.88 ms against 1.04 ms, 93 columns 1.32 against 1.49 ms.
-template <int KBS_, int KQ_, int KR_, uint32_t NA_, uint32_t NQ_, int DW_, int WW_, int MAXG_, bool PAIR_ = false>
+// LISTED: also built for lists of column tiles, whose widths are 64, 128 and 208.
+template <int KBS_, int KQ_, int KR_, uint32_t NA_, uint32_t NQ_, int DW_, int WW_, int MAXG_, bool LISTED_, bool PAIR_ = false>
 struct Cfg {
-  static constexpr bool PAIR = PAIR_;
+  static constexpr bool PAIR = PAIR_, LISTED = LISTED_;
   static constexpr uint32_t KBS = KBS_, KQ = KQ_, KR = KR_, NA = NA_, NQ = NQ_, DW = DW_, WW = WW_, MAXG = MAXG_;
   static constexpr uint32_t THREADS = (ISSUE_WARPS + DW + WW) * 32;
   static constexpr uint32_t RAW_STAGE = 2 * TM * KR;  // lo and hi tiles
@@ -141,12 +142,12 @@ struct Cfg {
 };
 // By tile width. Narrow tiles are bound by the database bytes and by the MMA warp's pace per stage: long
 // stages and eight widening warps. From 129 columns on TMEM leaves room for shorter stages only.
-using Cfg64 = Cfg<4, 4, 128, 2, 4, 4, 8, 4, true>;
-using Cfg96 = Cfg<2, 2, 128, 2, 4, 4, 8, 6, true>;
-using Cfg128 = Cfg<2, 2, 128, 4, 4, 4, 8, 8>;
-using Cfg160 = Cfg<2, 2, 128, 3, 3, 4, 8, 10>;
-using Cfg192 = Cfg<1, 2, 64, 3, 3, 8, 4, 6>;
-using Cfg208 = Cfg<1, 2, 64, 3, 3, 8, 4, 7>;
+using Cfg64 = Cfg<4, 4, 128, 2, 4, 4, 8, 4, true, true>;
+using Cfg96 = Cfg<2, 2, 128, 2, 4, 4, 8, 6, false, true>;
+using Cfg128 = Cfg<2, 2, 128, 4, 4, 4, 8, 8, true>;
+using Cfg160 = Cfg<2, 2, 128, 3, 3, 4, 8, 10, false>;
+using Cfg192 = Cfg<1, 2, 64, 3, 3, 8, 4, 6, false>;
+using Cfg208 = Cfg<1, 2, 64, 3, 3, 8, 4, 7, true>;
 static_assert(Cfg64::TN >= 64 && Cfg96::TN >= 96 && Cfg128::TN >= 128 && Cfg160::TN >= 160 && Cfg192::TN >= 192 && Cfg208::TN >= MAX_TN, "");
 static_assert(Cfg64::raw_stages(64) >= 2 && Cfg96::raw_stages(96) >= 2 && Cfg128::raw_stages(128) >= 2 && Cfg160::raw_stages(160) >= 2 &&
                   Cfg192::raw_stages(192) >= 2 && Cfg208::raw_stages(208) >= 2,
@@ -675,7 +676,7 @@ cudaError_t ready() {
   };
   set(reinterpret_cast<const void*>(&gemm_ts_kernel<F, false, false>));
   set(reinterpret_cast<const void*>(&gemm_ts_kernel<F, false, true>));
-  set(reinterpret_cast<const void*>(&gemm_ts_kernel<F, true, false>));
+  if constexpr (F::LISTED) set(reinterpret_cast<const void*>(&gemm_ts_kernel<F, true, false>));
   return e;
 }
 
@@ -718,9 +719,14 @@ int launch_ts(const TsMaps& m, TsParams& p, uint32_t ctas, uint32_t split, cudaS
     ++cfg.numAttrs;
   }
   cfg.attrs = at;
-  IPC_CUDA_TRY(cudaLaunchKernelEx(
-      &cfg, p.col_tiles ? gemm_ts_kernel<F, true, false> : split > 1 ? gemm_ts_kernel<F, false, true> : gemm_ts_kernel<F, false, false>,
-      m, p));
+  auto* kernel = split > 1 ? gemm_ts_kernel<F, false, true> : gemm_ts_kernel<F, false, false>;
+  if constexpr (F::LISTED) {
+    if (p.col_tiles) kernel = gemm_ts_kernel<F, true, false>;
+  } else if (p.col_tiles) {
+    set_error("tcgen05 ring GEMM: no form for listed tiles of this width");
+    return IPC_EINVAL;
+  }
+  IPC_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, m, p));
   return IPC_OK;
 }
 

@@ -50,3 +50,51 @@ def test_int8_tables_keep_their_key(torch, tmp_path):
         ipc.ipc_serve_stop(ctx)
     finally:
         ipc.ipc_destroy(ctx)
+
+
+@pytest.mark.parametrize("path,rows", [("tc", 5000), ("tcg", 5000), ("tc", 20000)])
+def test_every_tile_width_of_the_loop(torch, tmp_path, path, rows):
+    """Every tcgen05 variant (tiles of 256, 128, 208 and 64 columns) serves the same requests: 18 queries x 31
+    rotations in a pool of 768 columns, of which 208 does not divide (the last tile reaches past it), alone and
+    beside others, several tiles a CTA. Equal to the shares of the same queries submitted alone."""
+    ipc = lib()
+    gal = path == "tcg"
+    w = synth.Workload("widths", s=rows, Q=39, planted=5, seed=0x71D5 + rows)
+    code, mask = query_shares_gpu(w, galois_shares=gal)
+    sizes = [18, 5, 8, 3, 5]
+    cuts = np.cumsum([0] + sizes)
+
+    def run(variant):
+        ctx = make_ctx(w, path=path, chunk_rows=4096 if rows < 20000 else 0, max_queries=18)
+        try:
+            load_workload(ctx, w, galois_shares=gal)
+            if variant:
+                _start(ctx, 18, tmp_path / f"{variant}.json", variant)
+            shares = []
+            for burst in ([0], [1, 2, 3], [4]):
+                ids = []
+                for i in burst:
+                    part = [[v[j, cuts[i]:cuts[i + 1]].contiguous() for j in range(3)] for v in (code, mask)]
+                    if variant:
+                        part = [[t.cpu().numpy() for t in v] for v in part]
+                        ids.append((ipc.ipc_serve_submit(ctx, *part, sizes[i]), i))
+                    else:
+                        ids.append((ipc.submit_queries(ctx, *part, sizes[i], 1), i))
+                for rid, i in ids:
+                    sh = np.zeros((3, sizes[i]), np.uint8)
+                    ipc.fetch_bit_shares(ctx, rid, sh, sizes[i], 60000)
+                    ipc.ipc_release(ctx, rid)
+                    shares.append((rid, sh))
+            steps = ipc.ipc_serve_stats(ctx)["variant_steps"] if variant else None
+            return shares, steps
+        finally:
+            ipc.ipc_destroy(ctx)
+
+    want, _ = run(None)
+    bits = np.concatenate([s[0] ^ s[1] ^ s[2] for _, s in want])
+    assert np.nonzero(bits)[0].tolist() == sorted(w.planted_set())
+    for k, variant in enumerate(("tc256", "tc128", "tc208", "tc64")):
+        got, steps = run(variant)
+        assert [s > 0 for s in steps] == [i == k for i in range(4)]
+        for (rid, sh), (rid2, sh2) in zip(got, want):
+            assert rid == rid2 and (sh == sh2).all(), (variant, rid)
