@@ -513,8 +513,8 @@ extern "C" int submit_queries(ipc_ctx* c, const uint16_t* const code[3], const u
   const bool fused = c->cfg.fused != 0;
   // tcgen05 paths: the three parties' Z_2^16 GEMMs are launched together, on one stream. Chunks on two
   // streams put two query operands in L2 at once: 64.6 against 62.3 ms a step of 100,000 rows x 992
-  // columns. The Z_2^32 GEMMs go on the party streams, where each fills the last round of the one before:
-  // 20.6 against 21.3 ms a ConstLift step of 30,000 x 496 on one stream.
+  // columns. The Z_2^32 GEMMs go on the party streams, where each fills the last rounds of the others, or
+  // all on the first one.
   const bool joint = !fused && c->qsz == 2;
   if (joint) {
     for (int i = 1; i < 3; ++i) {
@@ -578,6 +578,7 @@ extern "C" int submit_queries(ipc_ctx* c, const uint16_t* const code[3], const u
       // seeds make its zero share vanish
       RingGemm g[RING_GEMM_PASSES];
       uint32_t n_pass = 0;
+      const bool in_turn = c->cfg.lift && ring_gemm_tc32_in_turn(2, ch.rows, N, l);
       for (int i = 0; i < (c->cfg.lift ? 3 : 1); ++i) SUB_TRY(cudaStreamWaitEvent(c->sp[i], c->ev_cmp[set], 0));
       for (int vec = 0; vec < 2; ++vec)
         for (int i = 0; i < 3; ++i) {
@@ -596,7 +597,7 @@ extern "C" int submit_queries(ipc_ctx* c, const uint16_t* const code[3], const u
             }
             SUB_RC(ring_gemm_tc32(2, x8, ch.rows, b4, N, n_pad, l, sl.tags, c->cfg.seeds[i], c->cfg.seeds[prev],
                                   static_cast<uint32_t>(vec), reinterpret_cast<uint32_t*>(zo), ldz, ch.row0,
-                                  c->sp[i]));
+                                  in_turn ? 1 : 3, c->sp[in_turn ? 0 : i]));
             continue;
           }
           g[n_pass++] = RingGemm{{i8p(plane(c, ch, i, vec, 0)), i8p(plane(c, ch, other, vec, 0))},

@@ -67,7 +67,6 @@ constexpr int ISSUE_WARPS = 4;
 constexpr uint32_t MAX_NR = 8;        // raw stages at most
 constexpr uint32_t SMEM_MAX = 231424;  // dynamic shared memory, leaving room for the static words
 constexpr uint32_t A_COLS = 32;       // TMEM columns of a widened k-block: lo 16, hi 16 (two fp16 a column)
-constexpr uint64_t L2_QUERY_BYTES = 112ull << 20;  // query operands that stay in L2 beside the database
 constexpr double LAUNCH_ROUNDS = 32;  // of the chip, of a launch whose passes' query operands don't fit the L2
 constexpr uint32_t MAX_TN = 208;      // 2 x 208 accumulator columns leave three widened k-blocks
 

@@ -7,6 +7,7 @@
 namespace ipc {
 
 constexpr uint32_t RING_GEMM_PASSES = 6;
+constexpr uint64_t L2_QUERY_BYTES = 112ull << 20;  // query operands that stay in L2 beside the database
 
 // One ring GEMM of a launch: z = [x[0] | x[1]] . b + zero share (segments = 2) or x[0] . b (segments = 1).
 struct RingGemm {

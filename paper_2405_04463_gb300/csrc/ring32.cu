@@ -17,6 +17,7 @@
 #include <string>
 #include <type_traits>
 
+#include "gemm_ts.cuh"
 #include "tcgen05_ts.cuh"
 
 namespace ipc {
@@ -151,11 +152,12 @@ __global__ void prep_query32_kernel(const uint32_t* __restrict__ y, uint64_t pla
 }
 
 // ----------------------------------- A3 -----------------------------------
-// One CTA per tile of 128 database rows x tn query columns. With four balanced limbs per operand
+// One CTA per tile of 128 database rows x nw query columns (the launch's columns dealt out in 16-column units,
+// so that tiles differ by one unit and none computes padding). With four balanced limbs per operand
 // z = sum over s of 2^(8s) S_s, S_s the sum of the limb products x_a y_b, a + b = s (ten per k; products
 // with a + b > 3 vanish mod 2^32). The database limbs are widened in registers and stored to tensor
 // memory, as in the 16-bit kernel, and the query tiles of a stage lie one under the other in shared
-// memory, so that one MMA of N = 2 tn multiplies a limb with two of them; its D is a pair of neighbouring
+// memory, so that one MMA of N = 2 nw multiplies a limb with two of them; its D is a pair of neighbouring
 // accumulators [S_0 | S_1 | S_2 | S_3]:
 //     H:  [S_2 | S_3] += x_0 [y_2 | y_3], x_1 [y_1 | y_2], x_2 [y_0 | y_1];  S_3 += x_3 y_0
 //     Lo: [S_0 | S_1] += x_0 [y_0 | y_1];  S_1 += x_1 y_0
@@ -166,7 +168,7 @@ __global__ void prep_query32_kernel(const uint32_t* __restrict__ y, uint64_t pla
 // earlier form kept both operands in shared memory, drained every 64 k and needed two passes over K for
 // tiles of 256 columns, because four accumulators of that width do not fit the 512 TMEM columns; with A
 // in tensor memory narrow MMAs run at the same rate, and 96 columns leave room for two widened k-blocks.
-// 65,536 rows x 992 columns (K = 25,600): 21.6 ms against 22.7 ms; 30,000 x 496: 5.26 against 6.09 ms;
+// 65,536 rows x 992 columns (K = 25,600): 21.6 ms against 22.7 ms; 30,000 x 496: 5.1 against 6.07 ms;
 // 19,456 x 96 (a tile per SM): 0.59 against 1.60 ms; 1,000 x 31: 0.053 against 1.51 ms. Two warps that
 // issue, one for H and one for Lo, take 5.95 ms at 30,000 x 496.
 constexpr int TM = 128, KB = 32;
@@ -180,16 +182,19 @@ constexpr uint32_t A_COLS = 64;        // TMEM columns of a widened k-block: fou
 constexpr uint32_t SMEM_MAX = 231424;
 constexpr uint32_t MAX_TN = 96, MAX_SPLIT = 8;
 constexpr uint32_t DW = 8, WW = 8, MAXG = 3, ISSUE_WARPS = 4, THREADS = (ISSUE_WARPS + DW + WW) * 32;
+constexpr uint32_t NA3_TN = 80;        // up to here the 512 TMEM columns hold three widened k-blocks beside the accumulators
 constexpr uint32_t MAX_NA = 3, NUM_BARS = 2 * NQ + 2 * MAX_NA + 2 * MAX_NR + 6;
 static_assert(MAX_TN <= MAXG * 16 * (DW / 4) && WW == 4 * KBR, "a drain thread's columns; a widening group per k-block of a raw stage");
 
 struct Maps32 {
-  CUtensorMap b[4];     // query limbs [n_pad][K], fp16
+  CUtensorMap b[2][4];  // query limbs [n_pad][K], fp16: boxes of tn columns, and of tn - 16
   CUtensorMap x[2][4];  // database limbs of the two K segments, [x_rows][l] int8
 };
 
 struct Tc32Params {
-  uint32_t n_cols, x_rows, tn, nr, n_ct, n_rt;
+  uint32_t n_cols, x_rows;
+  uint32_t tn;  // columns of the widest tiles; the others have 16 less
+  uint32_t nr, n_ct, n_rt;
   uint32_t segs, kb_seg;  // K segments; k-blocks of one
   const uint32_t* col_tags;
   uint64_t seed_own, seed_prev;
@@ -205,32 +210,14 @@ struct Tc32Params {
 // Every wait is bounded (2 s, or sooner once another role has failed); a failed CTA raises the status word,
 // lets its copies and MMAs finish, frees its tensor memory and stores nothing.
 template <uint32_t NA, bool SPLIT>
-__global__ void __launch_bounds__(THREADS, 1)
-    gemm_tc32_kernel(const __grid_constant__ Maps32 maps, const __grid_constant__ Tc32Params p) {
+__device__ __forceinline__ void tc32_tile(const Maps32& maps, const Tc32Params& p, uint32_t q0, uint32_t d0, uint32_t nw,
+                                          uint32_t rank, uint32_t n_rank) {
   constexpr uint32_t LEAD = NA, DT = DW * 32;
   static_assert(HP - LOFF >= LEAD && LOFF >= LEAD && LP % HP == 0 && NQ * KBR >= LEAD, "drains apart");
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ uint32_t s_abort;
-  const uint32_t tn = p.tn, q_tile = tn * 128, q_stage = 4 * q_tile;
-  uint32_t rank = 0, n_rank = 1;
-  if (SPLIT) {
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_rank));
-  }
-  // the tile: bands of up to 8 column tiles, all row tiles of a band before the next
-  constexpr uint32_t kBand = 8;
-  uint32_t q0, d0, nw;
-  {
-    const uint32_t lin = blockIdx.x / n_rank;
-    const uint32_t band = lin / (kBand * p.n_rt), c0 = band * kBand;
-    const uint32_t width = p.n_ct - c0 < kBand ? p.n_ct - c0 : kBand;
-    const uint32_t in_band = lin - band * kBand * p.n_rt, ct = c0 + in_band % width;
-    const uint32_t units = (p.n_cols + 15) / 16, base = units / p.n_ct, rem = units % p.n_ct;
-    q0 = 16 * (ct * base + (ct < rem ? ct : rem));
-    nw = 16 * (base + (ct < rem ? 1 : 0));
-    d0 = in_band / width * TM;
-  }
+  const uint32_t q_tile = nw * 128, q_stage = 4 * q_tile;
   const uint32_t k_units = p.segs * p.kb_seg / KB_UNIT;
   const uint32_t kb0 = SPLIT ? k_units * rank / n_rank * KB_UNIT : 0;
   const uint32_t nst = (SPLIT ? k_units * (rank + 1) / n_rank : k_units) * KB_UNIT - kb0;  // stages: one k-block each
@@ -276,7 +263,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = s_tmem, tH = tmem + 2 * tn, tA = tmem + 4 * tn;
+  const uint32_t tmem = s_tmem, tH = tmem + 2 * nw, tA = tmem + 4 * nw;
   auto all_wait = [&](uint32_t bar, uint32_t par) {
     return __all_sync(0xFFFFFFFFu, mbar_wait(bar, par, p.status, abort)) != 0;
   };
@@ -309,7 +296,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int32_t k = k_of(kb, seg), kx = k + static_cast<int32_t>(seg * p.kb_seg * KB);
         mbar_expect_tx(full, q_stage);
 #pragma unroll
-        for (uint32_t t = 0; t < 4; ++t) tma_load(base + t * q_tile, &maps.b[t], kx, static_cast<int32_t>(q0), full);
+        for (uint32_t t = 0; t < 4; ++t) tma_load(base + t * q_tile, &maps.b[nw != p.tn][t], kx, static_cast<int32_t>(q0), full);
       }
       __syncwarp();
       ++issued;
@@ -321,8 +308,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else if (warp == 1) {
     // -------------------------------- MMA issuer --------------------------------
-    const uint32_t id1 = (1u << 4) | ((tn >> 3) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
-    const uint32_t id2 = (1u << 4) | ((tn >> 2) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
+    const uint32_t id1 = (1u << 4) | ((nw >> 3) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
+    const uint32_t id2 = (1u << 4) | ((nw >> 2) << 17) | (static_cast<uint32_t>(TM >> 4) << 24);
     auto wait_stage = [&](uint32_t G) { return all_wait(a_full + 8 * stage_of<NA>(G), phase_of<NA>(G)); };
     auto free_stage = [&](uint32_t G) {
       if (G % KBR == KBR - 1) umma_commit(q_empty + 8 * stage_of<NQ>(G / KBR));
@@ -338,7 +325,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           umma_ts(tH, x, sdesc128(b + 2 * q_tile), id2, !(opens && ks == 0));  // x_0 [y_2 | y_3]
           umma_ts(tH, x + 16, sdesc128(b + q_tile), id2, true);                // x_1 [y_1 | y_2]
           umma_ts(tH, x + 32, sdesc128(b), id2, true);                         // x_2 [y_0 | y_1]
-          umma_ts(tH + tn, x + 48, sdesc128(b), id1, true);                    // x_3 y_0
+          umma_ts(tH + nw, x + 48, sdesc128(b), id1, true);                    // x_3 y_0
         }
         if ((G + 1) % HP == 0 || G + 1 == nst) umma_commit(h_full);
         if (frees) free_stage(G);
@@ -353,7 +340,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (uint32_t ks = 0; ks < KB / 16; ++ks) {
           const uint32_t b = q + 32u * ks, x = a + 8 * ks;
           umma_ts(tmem, x, sdesc128(b), id2, !(opens && ks == 0));  // x_0 [y_0 | y_1]
-          umma_ts(tmem + tn, x + 16, sdesc128(b), id1, true);       // x_1 y_0
+          umma_ts(tmem + nw, x + 16, sdesc128(b), id1, true);       // x_1 y_0
         }
         if (frees) free_stage(G);
         if ((G + 1) % LP == LOFF || G + 1 == nst) umma_commit(l_full);
@@ -484,7 +471,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (g < ng) {
           uint32_t a[16], b[16];
           tmem_ld16(t + 16 * g, a);
-          tmem_ld16(t + tn + 16 * g, b);
+          tmem_ld16(t + nw + 16 * g, b);
           tmem_wait_ld();
           if (g == ng - 1) {  // the last of this warp's columns is in registers
             fence_before();
@@ -501,7 +488,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     bool ok = true;
     for (uint32_t s = 1; s <= nst && ok; ++s) {
       if (s % HP == 0 || s == nst)
-        ok = drain(h_full, h_per++ & 1u, t0 + 2 * tn, h_empty, [&](uint32_t g, const uint32_t (&a)[16], const uint32_t (&b)[16]) {
+        ok = drain(h_full, h_per++ & 1u, t0 + 2 * nw, h_empty, [&](uint32_t g, const uint32_t (&a)[16], const uint32_t (&b)[16]) {
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
             const uint32_t u = add16x2(low16x2<1>(a[2 * k], a[2 * k + 1]), low16x2<256>(b[2 * k], b[2 * k + 1]));
@@ -519,7 +506,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     // ---- epilogue: the sums through the (now idle) query ring, then four rows of a column at a time ----
     if (!named_sync_or(1, DT, *abort != 0)) {
-      uint32_t* zs = reinterpret_cast<uint32_t*>(smem);  // [tn][TM]
+      uint32_t* zs = reinterpret_cast<uint32_t*>(smem);  // [nw][TM]
       const uint32_t row = 32 * (warp & 3u) + lane;
 #pragma unroll
       for (uint32_t k = 0; k < 16 * MAXG; ++k)
@@ -559,6 +546,33 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
+template <bool SPLIT>
+__global__ void __launch_bounds__(THREADS, 1)
+    gemm_tc32_kernel(const __grid_constant__ Maps32 maps, const __grid_constant__ Tc32Params p) {
+  uint32_t rank = 0, n_rank = 1;
+  if (SPLIT) {
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_rank));
+  }
+  // the tile, nw columns wide: bands of up to 8 column tiles, all row tiles of a band before the next
+  constexpr uint32_t kBand = 8;
+  uint32_t q0, d0, nw;
+  {
+    const uint32_t lin = blockIdx.x / n_rank;
+    const uint32_t band = lin / (kBand * p.n_rt), c0 = band * kBand;
+    const uint32_t width = p.n_ct - c0 < kBand ? p.n_ct - c0 : kBand;
+    const uint32_t in_band = lin - band * kBand * p.n_rt, ct = c0 + in_band % width;
+    const uint32_t units = (p.n_cols + 15) / 16, base = units / p.n_ct, rem = units % p.n_ct;
+    q0 = 16 * (ct * base + (ct < rem ? ct : rem));
+    nw = 16 * (base + (ct < rem ? 1 : 0));
+    d0 = in_band / width * TM;
+  }
+  if (nw > NA3_TN)
+    tc32_tile<2, SPLIT>(maps, p, q0, d0, nw, rank, n_rank);
+  else
+    tc32_tile<3, SPLIT>(maps, p, q0, d0, nw, rank, n_rank);
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 uint32_t cdiv(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
@@ -567,10 +581,8 @@ uint32_t cdiv(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
 uint32_t g_at_once[64][MAX_SPLIT + 1];
 
 cudaError_t ready() {
-  const void* k[4] = {reinterpret_cast<const void*>(&gemm_tc32_kernel<2, false>),
-                      reinterpret_cast<const void*>(&gemm_tc32_kernel<2, true>),
-                      reinterpret_cast<const void*>(&gemm_tc32_kernel<3, false>),
-                      reinterpret_cast<const void*>(&gemm_tc32_kernel<3, true>)};
+  const void* k[2] = {reinterpret_cast<const void*>(&gemm_tc32_kernel<false>),
+                      reinterpret_cast<const void*>(&gemm_tc32_kernel<true>)};
   cudaError_t e = load_kernels({reinterpret_cast<const void*>(&prep_query32_kernel)});
   for (const void* f : k)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
@@ -588,28 +600,36 @@ cudaError_t ready() {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, gemm_tc32_kernel<2, true>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, gemm_tc32_kernel<true>, &cfg);
     g_at_once[dev][s] = e == cudaSuccess ? static_cast<uint32_t>(n) * s : 0;
   }
   return e;
 }
 
-// Column tiles and parts of K with the shortest estimate, as for the 16-bit kernel: rounds of the chip x
-// (k-blocks of a CTA x cycles of one + a tile's start and end). A k-block takes 10 cycles a column, and at
-// least 650 at small widths (the raw copies and the widening). 496 columns as six tiles of up to 96 take
-// 5.53 ms, as seven of up to 80, which leave room for a third widened stage, 5.44 ms (30,000 rows, sustained).
-void pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t kb_total, uint32_t& n_ct, uint32_t& split) {
+// Column tiles and parts of K with the shortest estimate. A tile of w columns takes 68 + 9.9 w cycles a k-block,
+// a line through launches of the measured widths, and at least 650 (the raw copies and the widening). Its
+// tiles have base 16-column units or one more. Few rounds of the chip end together where all tiles are equal;
+// unequal ones fill half a round more than their number, but no round is shorter than the narrowest tile or
+// longer than the widest. `together` launches fill each other's last rounds. Then the parts of K, each with a
+// start and an end. Measured, tiles of two widths against equal ones with padding: 30,000 rows x 496 columns
+// 5.1-5.4 ms against 5.34-5.5, 17,000 x 372 2.14 against 2.38, 8,000 x 1,240 3.28 against 3.40.
+void pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t kb_total, uint32_t together, uint32_t& n_ct, uint32_t& split) {
   int dev = 0;
   const uint32_t* at_once = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_at_once[dev] : nullptr;
   const double sms = sm_count_current();
   const uint32_t units = cdiv(n_cols, 16), least = cdiv(units, MAX_TN / 16);
+  auto cycles = [](uint32_t w) { return std::max(650.0, 68 + 9.9 * 16 * w); };
   double best = 1e300;
-  for (uint32_t t = least; t <= least + 2 && t <= units; ++t) {
-    const double kb_cycles = std::max(650.0, 10.6 * 16 * cdiv(units, t)), ctas = static_cast<double>(t) * row_tiles;
+  for (uint32_t t = least; t <= least + 3 && t <= units; ++t) {
+    const uint32_t base = units / t, rem = units % t;
+    const double ctas = static_cast<double>(t) * row_tiles * together, most = cycles(base + (rem > 0)),
+                 mean = (rem * cycles(base + 1) + (t - rem) * cycles(base)) / t;
     for (uint32_t s = 1; s <= MAX_SPLIT && s <= kb_total / KB_UNIT; ++s) {
       if (s > 1 && (!at_once || at_once[s] == 0)) continue;
-      const double rounds = ctas * s / (s == 1 ? sms : at_once[s]);
-      const double cost = (rounds < 4 ? std::ceil(rounds) : rounds + 0.5) * (kb_cycles * kb_total / s + (s == 1 ? 10000 : 14000));
+      const double rounds = ctas * s / (s == 1 ? sms : at_once[s]), whole = std::ceil(rounds);
+      double tiles = (rounds + 0.5) * mean;
+      if (rounds < 8) tiles = std::min(std::max(rem ? tiles : 0.0, whole * cycles(base)), whole * most);
+      const double cost = tiles * kb_total / s + whole * (s == 1 ? 10000 : 14000);
       if (cost < best * 0.999) {
         best = cost;
         n_ct = t;
@@ -619,7 +639,6 @@ void pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t kb_total, uint32_t
   }
 }
 
-template <uint32_t NA>
 int launch_tc32(const Maps32& m, const Tc32Params& p, uint32_t split, uint32_t smem, cudaStream_t stream) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(p.n_ct * p.n_rt * split);
@@ -634,7 +653,7 @@ int launch_tc32(const Maps32& m, const Tc32Params& p, uint32_t split, uint32_t s
     ++cfg.numAttrs;
   }
   cfg.attrs = at;
-  IPC_CUDA_TRY(cudaLaunchKernelEx(&cfg, split > 1 ? gemm_tc32_kernel<NA, true> : gemm_tc32_kernel<NA, false>, m, p));
+  IPC_CUDA_TRY(cudaLaunchKernelEx(&cfg, split > 1 ? gemm_tc32_kernel<true> : gemm_tc32_kernel<false>, m, p));
   return IPC_OK;
 }
 
@@ -647,11 +666,22 @@ int ring_gemm_tc32_ready() {
   return IPC_OK;
 }
 
+// Whether a chunk's Z_2^32 GEMMs run best one after another: where two of their query operands do not fit the
+// L2 together, unless a launch has so few rounds of the chip that their last ones weigh more. Requests of 30,000
+// rows x 496 columns without lifting, sustained: 32.0 ms on one stream, 33.8 ms on the party streams; 65,536 x
+// 992: 132 and 144 ms; 65,536 x 155 with ConstLift: 14.1 and 13.8 ms.
+bool ring_gemm_tc32_in_turn(uint32_t segments, size_t x_rows, uint32_t n_cols, uint32_t l) {
+  const double rounds = static_cast<double>(cdiv(n_cols, MAX_TN)) * cdiv(static_cast<uint32_t>(x_rows), TM) / sm_count_current();
+  return 2 * 8ull * segments * l * n_cols > L2_QUERY_BYTES && rounds >= 2;
+}
+
 // segments: 2 for K = 2l over [x[0..3] | x[4..7]] (ABY3 replicated sharing, x[4..7] the
-// previous party's component), 1 for K = l over x[0..3] alone. K must be a multiple of 256.
+// previous party's component), 1 for K = l over x[0..3] alone. K must be a multiple of 256. together: like
+// launches in flight at the same time, this one among them.
 int ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], size_t x_rows, const uint16_t* const b[4],
                    uint32_t n_cols, uint32_t n_pad, uint32_t l, const uint32_t* col_tags, uint64_t seed_own,
-                   uint64_t seed_prev, uint32_t vec, uint32_t* z, size_t ldz, uint64_t row0, cudaStream_t stream) {
+                   uint64_t seed_prev, uint32_t vec, uint32_t* z, size_t ldz, uint64_t row0, uint32_t together,
+                   cudaStream_t stream) {
   if (segments != 1 && segments != 2) {
     set_error("Z_2^32 ring GEMM: one or two K segments");
     return IPC_EINVAL;
@@ -674,7 +704,7 @@ int ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], size_t x_rows, c
   p.n_rt = static_cast<uint32_t>((x_rows + TM - 1) / TM);
   p.n_ct = 1;
   uint32_t split = 1;
-  pick_shape(n_cols, p.n_rt, segments * l / KB, p.n_ct, split);
+  pick_shape(n_cols, p.n_rt, segments * l / KB, together, p.n_ct, split);
   p.tn = 16 * cdiv(cdiv(n_cols, 16), p.n_ct);
   const uint32_t q_stage = 4 * p.tn * 128;
   p.nr = std::min(MAX_NR, (SMEM_MAX - 1024 - 8 * NUM_BARS - NQ * q_stage) / RAW_STAGE);
@@ -682,7 +712,8 @@ int ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], size_t x_rows, c
   Maps32 m;
   int rc;
   for (int i = 0; i < 4; ++i) {
-    if ((rc = make_map_f16k64(&m.b[i], b[i], static_cast<uint64_t>(segments) * l, n_pad, p.tn)) ||
+    if ((rc = make_map_f16k64(&m.b[0][i], b[i], static_cast<uint64_t>(segments) * l, n_pad, p.tn)) ||
+        (rc = make_map_f16k64(&m.b[1][i], b[i], static_cast<uint64_t>(segments) * l, n_pad, std::max(16u, p.tn - 16))) ||
         (rc = make_map_raw(&m.x[0][i], x[i], l, x_rows, KR, TM)) ||
         (rc = make_map_raw(&m.x[1][i], x[segments == 2 ? 4 + i : i], l, x_rows, KR, TM)))
       return rc;
@@ -699,8 +730,7 @@ int ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], size_t x_rows, c
   p.ldz = ldz;
   p.row0 = row0;
   p.status = status_ptr();
-  return p.tn > 80 ? launch_tc32<2>(m, p, split, smem, stream)
-                   : launch_tc32<3>(m, p, split, smem, stream);
+  return launch_tc32(m, p, split, smem, stream);
 }
 
 int prep_query32(const uint32_t* y, uint64_t y_plane, uint32_t Q, const ipc_geom* g, uint32_t party,
@@ -795,6 +825,6 @@ extern "C" int ipc_ring_gemm_tc32(uint32_t segments, const int8_t* const x[8], s
     set_error("ipc_ring_gemm_tc32: l must be a multiple of 16");
     return IPC_EINVAL;
   }
-  return ring_gemm_tc32(segments, x, x_rows, b, n_cols, n_pad, l, col_tags, seed_own, seed_prev, vec, z, ldz, row0,
+  return ring_gemm_tc32(segments, x, x_rows, b, n_cols, n_pad, l, col_tags, seed_own, seed_prev, vec, z, ldz, row0, 1,
                         static_cast<cudaStream_t>(stream));
 }
