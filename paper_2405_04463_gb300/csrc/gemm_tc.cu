@@ -1,7 +1,8 @@
-// The fused chunk step (ipc_config.fused): the six ring GEMMs of a chunk (A3) tile by tile on the
-// 5th-generation tensor cores, each tile followed by its comparison phase (A4-A8), in one launch. Its
-// GEMM keeps both operands in shared memory and accumulators in tensor memory; the unfused steps use the
-// form with the database operand in tensor memory (gemm_ts.cu), which leaves no room for the comparison.
+// The ring GEMM (A3) on the 5th-generation tensor cores with both operands in shared memory and tiles of 256
+// query columns, in two forms: the fused chunk step (ipc_config.fused), a chunk's six ring GEMMs tile by tile,
+// each tile followed by its comparison phase (A4-A8), in one launch; and up to six ring GEMMs of a chunk
+// without the comparison, for the column counts whose last tile is nearly full, where the form with the
+// database operand in tensor memory (gemm_ts.cu, tiles of up to 208 columns) takes two tiles of about 128.
 //
 // The ring product is three limb products (Sec. 6.1):
 //     z = L + 256 C + r  (mod 2^16),  L = sum lo*lo',  C = sum (lo*hi' + hi*lo').
@@ -43,6 +44,7 @@
 // Every wait is bounded (2 s, or sooner once another role has failed); a failed CTA raises the
 // status word, lets its copies and MMAs finish, frees its tensor memory and stores nothing.
 #include "compare.cuh"
+#include "gemm_ts.cuh"
 #include "tcgen05.cuh"
 
 namespace ipc {
@@ -108,16 +110,20 @@ struct TcParams {
 // 128-row part) unit per drain thread, through the same part routine and gate numbering as the
 // stand-alone comparison kernel, its scratch in the Q ring (idle until the drain releases it).
 // The part roots are joined into 1,024-row block roots by or_join_parts afterwards.
-constexpr uint32_t NPASS = 6;
+constexpr uint32_t NPASS = RING_GEMM_PASSES;
 struct FuseMaps {
   CUtensorMap q[NPASS][2];  // query operand of pass ps (party ps / 2, vector ps % 2): lo, hi limbs
   CUtensorMap x[NPASS][2];  // database planes of component c, vector v at 2 c + v: lo, hi limbs
 };
 struct FuseParams {
   uint32_t n_ct;           // column tiles of the launch
+  uint32_t n_pass;         // six when fused
   uint16_t* z[NPASS];      // z of pass ps, [n_cols][ldz]
-  uint64_t seeds[3];       // seeds[j] shared by parties j and j + 1
-  cmp::Seeds keys;         // their round keys
+  uint32_t x0[NPASS], x1[NPASS];  // database planes of its two K segments (of its one, twice)
+  uint64_t seed_own[NPASS], seed_prev[NPASS];
+  uint32_t vec[NPASS];
+  // fused only:
+  cmp::Seeds keys;         // the round keys of the seeds shared by parties j and j + 1
   uint32_t thr_a;
   uint32_t* part_roots;    // [3][n_cols][ld_parts]: OR root of (column, row tile) of the chunk
   uint64_t ld_parts;
@@ -162,27 +168,30 @@ __device__ __noinline__ void fused_part_compare(const TcParams& p, const FusePar
   fp.part_roots[2 * plane + at] = root.c2;
 }
 
-template <int TN>
+template <int TN, bool FUSED>
 __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams& p, const FuseParams& fp) {
   using S = Shape<TN>;
   constexpr int B_BYTES = S::B_BYTES;
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ uint32_t s_abort;
-  // items: the six passes of each of this CTA's tiles, tile after tile
-  const uint32_t n_ct = fp.n_ct, n_tiles = n_ct * p.n_row_tiles;
-  const uint32_t my_tiles = n_tiles > blockIdx.x ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  if (my_tiles == 0) return;  // uniform for the CTA, before any barrier or allocation
-  const uint32_t my_items = my_tiles * NPASS;
+  // items: fused, the six passes of each of this CTA's tiles, tile after tile; else all tiles of a pass
+  // come before the next pass
+  const uint32_t n_ct = fp.n_ct, n_tiles = n_ct * p.n_row_tiles, n_work = FUSED ? n_tiles : n_tiles * fp.n_pass;
+  const uint32_t mine = n_work > blockIdx.x ? (n_work - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+  if (mine == 0) return;  // uniform for the CTA, before any barrier or allocation
+  const uint32_t my_items = FUSED ? mine * NPASS : mine;
   // A CTA takes tiles blockIdx.x + i gridDim.x of a linear order that walks bands of up to kBand column tiles,
   // all row tiles of a band before the next, so that the tiles in flight at once (one CTA per
   // SM) cover about 19 row tiles x 8 column tiles: each database tile is read by the band's
   // CTAs together and the band's query tiles stay in L2 while the rows stream past (with many
   // query columns the whole query operand is several times the L2).
   constexpr uint32_t kBand = 8;
-  auto coords = [&](uint32_t i, uint32_t& q0, uint32_t& d0) {
+  auto coords = [&](uint32_t i, uint32_t& q0, uint32_t& d0, uint32_t& ps) {
     const uint32_t n_rt = p.n_row_tiles;
-    const uint32_t lin = blockIdx.x + (i / NPASS) * gridDim.x;
+    uint32_t lin = blockIdx.x + (FUSED ? i / NPASS : i) * gridDim.x;
+    ps = FUSED ? i % NPASS : lin / n_tiles;
+    if (!FUSED) lin -= ps * n_tiles;
     const uint32_t band = lin / (kBand * n_rt), c0 = band * kBand;
     const uint32_t width = n_ct - c0 < kBand ? n_ct - c0 : kBand;
     const uint32_t in_band = lin - band * kBand * n_rt;
@@ -234,8 +243,8 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
       uint32_t issued = 0;
       bool ok = true;
       for (uint32_t i = 0; i < my_items && ok; ++i) {
-        uint32_t q0, d0;
-        coords(i, q0, d0);
+        uint32_t q0, d0, ps;
+        coords(i, q0, d0, ps);
         if (i > 0 && !mbar_wait(epi_done, (i - 1) & 1u, p.status, abort)) break;
         for (uint32_t kb = 0; kb < p.kb_total; ++kb) {
           const uint32_t G = i * p.kb_total + kb, s = G % QS;
@@ -244,8 +253,8 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
             break;
           }
           const uint32_t full = q_full + 8 * s, base = qring + s * S::Q_STAGE;
-          const CUtensorMap* mlo = &fm.q[i % NPASS][0];
-          const CUtensorMap* mhi = &fm.q[i % NPASS][1];
+          const CUtensorMap* mlo = &fm.q[ps][0];
+          const CUtensorMap* mhi = &fm.q[ps][1];
           mbar_expect_tx(full, 2 * B_BYTES);
           tma_load(base, mlo, static_cast<int32_t>(kb * KB), static_cast<int32_t>(q0), full);
           tma_load(base + B_BYTES, mhi, static_cast<int32_t>(kb * KB), static_cast<int32_t>(q0), full);
@@ -327,18 +336,17 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
     // k-block G + RS into raw stage G % RS once the warp has read k-block G from it.
     const uint32_t pl = static_cast<uint32_t>(warp - WIDEN_WARP0);  // 0: lo limbs, 1: hi limbs
     const uint32_t rf = r_full + 8 * RS * pl;
-    // the database planes of item i's two K segments: components ps / 2 and ps / 2 - 1 of the pass's vector
-    auto seg_maps = [&](uint32_t i, const CUtensorMap*& m0, const CUtensorMap*& m1) {
-      const uint32_t ps = i % NPASS, party = ps >> 1, vec = ps & 1u;
-      m0 = &fm.x[2 * party + vec][pl];
-      m1 = &fm.x[2 * ((party + 2) % 3) + vec][pl];
+    // the database planes of a pass's two K segments
+    auto seg_maps = [&](uint32_t ps, const CUtensorMap*& m0, const CUtensorMap*& m1) {
+      m0 = &fm.x[fp.x0[ps]][pl];
+      m1 = &fm.x[fp.x1[ps]][pl];
     };
     const CUtensorMap *map0, *map1;
     // the next raw copy (lane 0): k-block li_kb of item li, whose row offset li_d0 and tensor
     // maps are looked up once per item, so that a copy costs no division
-    uint32_t issued = 0, li = 0, li_kb = 0, li_q0 = 0, li_d0 = 0;
-    coords(0, li_q0, li_d0);
-    seg_maps(0, map0, map1);
+    uint32_t issued = 0, li = 0, li_kb = 0, li_q0 = 0, li_d0 = 0, li_ps = 0;
+    coords(0, li_q0, li_d0, li_ps);
+    seg_maps(li_ps, map0, map1);
     auto load_raw = [&](uint32_t G) {
       const uint32_t s = G % RS;
       const bool first = li_kb < p.kb_half;
@@ -349,8 +357,8 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
       if (++li_kb == p.kb_total) {
         li_kb = 0;
         if (++li < my_items) {
-          coords(li, li_q0, li_d0);
-          seg_maps(li, map0, map1);
+          coords(li, li_q0, li_d0, li_ps);
+          seg_maps(li_ps, map0, map1);
         }
       }
     };
@@ -446,10 +454,10 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
       // every drainer takes the same decision: the barrier returns whether any of them saw the
       // abort flag
       if (named_sync_or(1, DRAIN_THREADS, *abort != 0)) break;
-      uint32_t q0, d0;
-      coords(i, q0, d0);
-      const uint32_t ps = i % NPASS, party = ps >> 1, vec = ps & 1u;
-      const uint64_t seed_own = fp.seeds[party], seed_prev = fp.seeds[(party + 2) % 3];
+      uint32_t q0, d0, ps;
+      coords(i, q0, d0, ps);
+      const uint32_t vec = fp.vec[ps];
+      const uint64_t seed_own = fp.seed_own[ps], seed_prev = fp.seed_prev[ps];
       uint16_t* const zout = fp.z[ps];
       uint16_t* zs = reinterpret_cast<uint16_t*>(smem);  // [TN][TM]
       const uint32_t row = 32 * q + lane;
@@ -479,13 +487,16 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
                                    add2(acc.w, fo.w, fq.w));
         uint16_t* dst = zout + static_cast<uint64_t>(col) * p.ldz + r0;
         if (r0 + 8 <= p.x_rows) {
-          *reinterpret_cast<uint4*>(dst) = v;  // kept in L2: this CTA reads it back after the tile's last pass
+          if (FUSED)
+            *reinterpret_cast<uint4*>(dst) = v;  // kept in L2: this CTA reads it back after the tile's last pass
+          else
+            __stcs(reinterpret_cast<uint4*>(dst), v);  // streamed: z is read by a later kernel, not from L2
         } else {
           const uint32_t w[4] = {v.x, v.y, v.z, v.w};
           for (uint32_t e = 0; e < p.x_rows - r0; ++e) dst[e] = static_cast<uint16_t>(w[e >> 1] >> (16 * (e & 1)));
         }
       }
-      if (ps == NPASS - 1) {
+      if (FUSED && ps == NPASS - 1) {
         // ---- A4-A8 on the tile: its six z tiles are in global memory (L2), written by this
         // CTA's drainers; the barrier orders those stores before the reads below ----
         named_sync(1, DRAIN_THREADS);
@@ -508,10 +519,76 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_cmp_kernel(const __grid_constant__ FuseMaps fm, const __grid_constant__ TcParams p,
                     const __grid_constant__ FuseParams fp) {
-  gemm_tc_body<256>(fm, p, fp);
+  gemm_tc_body<256, true>(fm, p, fp);
+}
+
+__global__ void __launch_bounds__(THREADS, 1)
+    gemm_ss_kernel(const __grid_constant__ FuseMaps fm, const __grid_constant__ TcParams p,
+                   const __grid_constant__ FuseParams fp) {
+  gemm_tc_body<256, false>(fm, p, fp);
 }
 
 }  // namespace
+
+// Loads the kernel on this device (once).
+int ring_gemm_ss_ready() {
+  static PerDevice attr;
+  IPC_CUDA_TRY(attr.run([] {
+    return cudaFuncSetAttribute(gemm_ss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<256>::SMEM_BYTES);
+  }));
+  return IPC_OK;
+}
+
+// n_pass ring GEMMs with equal K segments over the same rows and columns in one persistent launch; arguments
+// checked by ring_gemm_ts.
+int ring_gemm_ss(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,
+                 const uint32_t* col_tags, size_t ldz, uint64_t row0, cudaStream_t stream) {
+  const uint32_t K = g[0].segments * l;
+  int rc = ring_gemm_ss_ready();
+  if (rc) return rc;
+  FuseMaps fm;
+  FuseParams fp{};
+  uint32_t nx = 0;
+  const int8_t* seen[NPASS][2];
+  auto x_map = [&](const int8_t* lo, const int8_t* hi, uint32_t& at) {
+    for (at = 0; at < nx; ++at)
+      if (seen[at][0] == lo && seen[at][1] == hi) return static_cast<int>(IPC_OK);
+    if (nx == NPASS) {
+      set_error("tcgen05 ring GEMM: too many database planes in one launch");
+      return static_cast<int>(IPC_EINVAL);
+    }
+    seen[nx][0] = lo;
+    seen[nx++][1] = hi;
+    const int e = make_map_i8(&fm.x[at][0], lo, l, x_rows, TM);
+    return e ? e : make_map_i8(&fm.x[at][1], hi, l, x_rows, TM);
+  };
+  for (uint32_t s = 0; s < n_pass; ++s) {
+    if ((rc = make_map_f16(&fm.q[s][0], g[s].b_lo, K, n_pad, 256)) || (rc = make_map_f16(&fm.q[s][1], g[s].b_hi, K, n_pad, 256)) ||
+        (rc = x_map(g[s].x_lo[0], g[s].x_hi[0], fp.x0[s])) ||
+        (rc = x_map(g[s].x_lo[g[s].segments - 1], g[s].x_hi[g[s].segments - 1], fp.x1[s])))
+      return rc;
+    fp.z[s] = g[s].z;
+    fp.seed_own[s] = g[s].seed_own;
+    fp.seed_prev[s] = g[s].seed_prev;
+    fp.vec[s] = g[s].vec;
+  }
+  fp.n_pass = n_pass;
+  fp.n_ct = (n_cols + 255) / 256;
+  TcParams p{};
+  p.n_cols = n_cols;
+  p.x_rows = static_cast<uint32_t>(x_rows);
+  p.kb_total = K / KB;
+  p.kb_half = l / KB;
+  p.n_row_tiles = static_cast<uint32_t>((x_rows + TM - 1) / TM);
+  p.col_tags = col_tags;
+  p.ldz = ldz;
+  p.row0 = row0;
+  p.status = status_ptr();
+  const uint32_t items = n_pass * fp.n_ct * p.n_row_tiles, sms = static_cast<uint32_t>(sm_count_current());
+  gemm_ss_kernel<<<items < sms ? items : sms, THREADS, Shape<256>::SMEM_BYTES, stream>>>(fm, p, fp);
+  IPC_CUDA_TRY(cudaGetLastError());
+  return IPC_OK;
+}
 
 // Loads the kernel on this device (once).
 int ring_gemm_compare_ready() {
@@ -570,7 +647,15 @@ int ring_gemm_compare_tc(uint32_t segments, const int8_t* const x_lo[6], const i
   FuseParams fp{};
   fp.n_ct = (n_cols + 255) / 256;
   for (uint32_t s = 0; s < NPASS; ++s) fp.z[s] = z[s];
-  for (int j = 0; j < 3; ++j) fp.seeds[j] = seeds[j];
+  fp.n_pass = NPASS;
+  for (uint32_t s = 0; s < NPASS; ++s) {
+    const uint32_t party = s / 2, prev = (party + 2) % 3;
+    fp.vec[s] = s % 2;
+    fp.x0[s] = s;
+    fp.x1[s] = 2 * prev + fp.vec[s];
+    fp.seed_own[s] = seeds[party];
+    fp.seed_prev[s] = seeds[prev];
+  }
   fp.keys = cmp::make_seeds(seeds);
   fp.thr_a = thr_a;
   fp.part_roots = part_roots;

@@ -739,8 +739,8 @@ uint32_t cdiv(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
 // At 1,000 rows x 4 columns splitting K by 8 gives 0.023 ms against 0.15 ms unsplit, at 1,000 x 279 0.042
 // against 0.085 ms with a guess of nine SMs in ten for clusters; 9,973 x 217 takes two tiles of 112 by 2
 // (0.31 ms; unsplit 0.40), 40,000 x 279 two tiles of 144 (0.67 ms; three of 96: 0.73).
-void pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t n_pass, uint32_t kb_total, uint32_t sms, uint32_t& n_ct,
-                uint32_t& split) {
+double pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t n_pass, uint32_t kb_total, uint32_t sms, uint32_t& n_ct,
+                  uint32_t& split) {
   int dev = 0;
   const uint32_t* at_once = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_at_once[dev] : nullptr;
   const uint32_t units = cdiv(n_cols, 16), least = cdiv(units, MAX_TN / 16);
@@ -758,13 +758,26 @@ void pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t n_pass, uint32_t k
       }
     }
   }
+  return best;
+}
+
+// The estimate of the form with both operands in shared memory, whose tiles are 256 columns wide and take 1,030
+// of these cycles a k-block: less than two tiles of 128 (1,127), more than one of 208 and a part of the next
+// columns'. So it pays from 241 to 256 columns, and at 500 where it saves a round. A request of 248 columns,
+// sustained: 65,536 rows of Galois-ring shares 5.64 ms with tiles of 128 and 5.38 ms so, replicated 10.63 and
+// 10.27 ms; 8,000 x 496 Galois 1.41 and 1.36 ms. 4 % must be gained to leave the estimates' errors behind.
+double ss_cost(uint32_t n_cols, uint32_t row_tiles, uint32_t n_pass, uint32_t kb_total, uint32_t sms) {
+  const double rounds = static_cast<double>(n_pass) * cdiv(n_cols, 256) * row_tiles / sms;
+  return (rounds < 8 ? std::ceil(rounds) : rounds + 0.5) * (1030.0 * kb_total + 10000) / 0.96;
 }
 
 int ring_gemm_ts_group(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,
                  const uint32_t* col_tags, size_t ldz, uint64_t row0, uint32_t list_cols, const uint32_t* col_tiles,
                  const uint32_t* n_col_list, cudaStream_t stream) {
   uint32_t kb_most = 0;
+  bool equal = true;
   for (uint32_t i = 0; i < n_pass; ++i) {
+    equal = equal && g[i].segments == g[0].segments;
     if (g[i].segments != 1 && g[i].segments != 2) {
       set_error("tcgen05 ring GEMM: one or two K segments");
       return IPC_EINVAL;
@@ -795,7 +808,9 @@ int ring_gemm_ts_group(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32
     }
   } else {
     p.n_col_tiles = 1;
-    pick_shape(n_cols, p.n_row_tiles, n_pass, kb_most, sms, p.n_col_tiles, split);
+    const double cost = pick_shape(n_cols, p.n_row_tiles, n_pass, kb_most, sms, p.n_col_tiles, split);
+    if (equal && ss_cost(n_cols, p.n_row_tiles, n_pass, kb_most, sms) < cost)
+      return ring_gemm_ss(n_pass, g, x_rows, n_cols, n_pad, l, col_tags, ldz, row0, stream);
     p.tn = 16 * cdiv(cdiv(n_cols, 16), p.n_col_tiles);
   }
   const uint32_t raw_cols = p.tn <= 64    ? Cfg64::KR
@@ -862,6 +877,7 @@ int ring_gemm_ts_group(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32
 }  // namespace
 
 int ring_gemm_ts_ready() {
+  if (const int rc = ring_gemm_ss_ready()) return rc;
   static PerDevice attr;
   IPC_CUDA_TRY(attr.run([] {
     cudaError_t e = ready<Cfg64>();

@@ -19,6 +19,11 @@ struct RingGemm {
   uint16_t* z;                      // [n_cols][ldz]
 };
 
+// The form with both operands in shared memory (gemm_tc.cu): passes of equal segments, tiles of 256 columns.
+int ring_gemm_ss_ready();
+int ring_gemm_ss(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,
+                 const uint32_t* col_tags, size_t ldz, uint64_t row0, cudaStream_t stream);
+
 // Loads every form of the kernel on this device (once). Loading one may wait for the work on the device, so
 // contexts call this when they are made; without it the first launch does.
 int ring_gemm_ts_ready();
