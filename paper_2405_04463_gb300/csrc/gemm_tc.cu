@@ -116,7 +116,9 @@ struct FuseMaps {
   CUtensorMap x[NPASS][2];  // database planes of component c, vector v at 2 c + v: lo, hi limbs
 };
 struct FuseParams {
-  uint32_t n_ct;           // column tiles of the launch
+  uint32_t n_ct;           // column tiles of the launch, or of the pool that a list selects from
+  const uint32_t* col_tiles;   // the column tiles to compute (device), or null: all of them
+  const uint32_t* n_col_list;  // their count (device)
   uint32_t n_pass;         // six when fused
   uint16_t* z[NPASS];      // z of pass ps, [n_cols][ldz]
   uint32_t x0[NPASS], x1[NPASS];  // database planes of its two K segments (of its one, twice)
@@ -177,7 +179,8 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
   __shared__ uint32_t s_abort;
   // items: fused, the six passes of each of this CTA's tiles, tile after tile; else all tiles of a pass
   // come before the next pass
-  const uint32_t n_ct = fp.n_ct, n_tiles = n_ct * p.n_row_tiles, n_work = FUSED ? n_tiles : n_tiles * fp.n_pass;
+  const bool listed = !FUSED && fp.col_tiles;
+  const uint32_t n_ct = listed ? *fp.n_col_list : fp.n_ct, n_tiles = n_ct * p.n_row_tiles, n_work = FUSED ? n_tiles : n_tiles * fp.n_pass;
   const uint32_t mine = n_work > blockIdx.x ? (n_work - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
   if (mine == 0) return;  // uniform for the CTA, before any barrier or allocation
   const uint32_t my_items = FUSED ? mine * NPASS : mine;
@@ -196,7 +199,7 @@ __device__ __forceinline__ void gemm_tc_body(const FuseMaps& fm, const TcParams&
     const uint32_t width = n_ct - c0 < kBand ? n_ct - c0 : kBand;
     const uint32_t in_band = lin - band * kBand * n_rt;
     const uint32_t ct = c0 + in_band % width;
-    q0 = ct * TN;
+    q0 = (listed ? fp.col_tiles[ct] : ct) * TN;
     d0 = (in_band / width) * TM;
   };
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -539,10 +542,11 @@ int ring_gemm_ss_ready() {
   return IPC_OK;
 }
 
-// n_pass ring GEMMs with equal K segments over the same rows and columns in one persistent launch; arguments
-// checked by ring_gemm_ts.
+// n_pass ring GEMMs with equal K segments over the same rows and columns, or a list of their 256-column tiles,
+// in one persistent launch; arguments checked by ring_gemm_ts_by.
 int ring_gemm_ss(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,
-                 const uint32_t* col_tags, size_t ldz, uint64_t row0, cudaStream_t stream) {
+                 const uint32_t* col_tags, size_t ldz, uint64_t row0, const uint32_t* col_tiles,
+                 const uint32_t* n_col_list, cudaStream_t stream) {
   const uint32_t K = g[0].segments * l;
   int rc = ring_gemm_ss_ready();
   if (rc) return rc;
@@ -574,6 +578,8 @@ int ring_gemm_ss(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_c
   }
   fp.n_pass = n_pass;
   fp.n_ct = (n_cols + 255) / 256;
+  fp.col_tiles = col_tiles;
+  fp.n_col_list = n_col_list;
   TcParams p{};
   p.n_cols = n_cols;
   p.x_rows = static_cast<uint32_t>(x_rows);
@@ -585,7 +591,7 @@ int ring_gemm_ss(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_c
   p.row0 = row0;
   p.status = status_ptr();
   const uint32_t items = n_pass * fp.n_ct * p.n_row_tiles, sms = static_cast<uint32_t>(sm_count_current());
-  gemm_ss_kernel<<<items < sms ? items : sms, THREADS, Shape<256>::SMEM_BYTES, stream>>>(fm, p, fp);
+  gemm_ss_kernel<<<items < sms && !col_tiles ? items : sms, THREADS, Shape<256>::SMEM_BYTES, stream>>>(fm, p, fp);
   IPC_CUDA_TRY(cudaGetLastError());
   return IPC_OK;
 }

@@ -83,7 +83,6 @@ struct TsParams {
   uint32_t kb_seg;             // k-blocks of a K segment, l / KB
   uint32_t n_col_tiles, n_row_tiles, n_pass;
   uint32_t pass_inner;         // the passes of a tile are neighbours (else all tiles of a pass come first)
-  uint32_t subs, list_cols;    // list mode: tiles per listed column tile, and its width
   const uint32_t* col_tiles;
   const uint32_t* n_col_list;
   const uint32_t* col_tags;
@@ -169,7 +168,7 @@ __global__ void __launch_bounds__(F::THREADS, 1)
   const uint32_t tn = p.tn, q_half = tn * 128, q_blk = 2 * q_half, q_stage = KQ / 2 * q_blk;
   uint32_t my_items = 1, n_ct = p.n_col_tiles;
   if (LIST) {
-    n_ct = *p.n_col_list * p.subs;
+    n_ct = *p.n_col_list;
     const uint32_t n_items = n_ct * p.n_row_tiles * p.n_pass;
     my_items = n_items > blockIdx.x ? (n_items - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
     if (my_items == 0) return;  // uniform for the CTA, before any barrier or allocation
@@ -203,7 +202,7 @@ __global__ void __launch_bounds__(F::THREADS, 1)
     const uint32_t in_band = lin - band * kBand * n_rt;
     const uint32_t ct = c0 + in_band % width;
     if (LIST) {
-      q0 = p.col_tiles[ct / p.subs] * p.list_cols + (ct % p.subs) * tn;
+      q0 = p.col_tiles[ct] * tn;
       nw = tn;
     } else {
       // the 16-column units of n_cols dealt out evenly: no tile computes more than its share of padding
@@ -799,18 +798,15 @@ int ring_gemm_ts_group(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32
   uint32_t split = 1;
   p.n_row_tiles = cdiv(static_cast<uint32_t>(x_rows), TM);
   if (col_tiles) {
-    p.list_cols = list_cols;
-    p.subs = cdiv(list_cols, MAX_TN);
-    p.tn = list_cols / p.subs;
-    if (p.tn % 16 != 0 || p.tn * p.subs != list_cols) {
-      set_error("tcgen05 ring GEMM: listed tiles divide into tiles of whole 16-column units");
-      return IPC_EINVAL;
-    }
+    // 256 columns: their own kernel, as two tiles of 128 they cost 10 % more
+    if (list_cols == 256)
+      return ring_gemm_ss(n_pass, g, x_rows, n_cols, n_pad, l, col_tags, ldz, row0, col_tiles, n_col_list, stream);
+    p.tn = list_cols;
   } else {
     p.n_col_tiles = 1;
     const double cost = pick_shape(n_cols, p.n_row_tiles, n_pass, kb_most, sms, p.n_col_tiles, split);
     if (equal && ss_cost(n_cols, p.n_row_tiles, n_pass, kb_most, sms) < cost)
-      return ring_gemm_ss(n_pass, g, x_rows, n_cols, n_pad, l, col_tags, ldz, row0, stream);
+      return ring_gemm_ss(n_pass, g, x_rows, n_cols, n_pad, l, col_tags, ldz, row0, nullptr, nullptr, stream);
     p.tn = 16 * cdiv(cdiv(n_cols, 16), p.n_col_tiles);
   }
   const uint32_t raw_cols = p.tn <= 64    ? Cfg64::KR

@@ -22,7 +22,8 @@ struct RingGemm {
 // The form with both operands in shared memory (gemm_tc.cu): passes of equal segments, tiles of 256 columns.
 int ring_gemm_ss_ready();
 int ring_gemm_ss(uint32_t n_pass, const RingGemm* g, size_t x_rows, uint32_t n_cols, uint32_t n_pad, uint32_t l,
-                 const uint32_t* col_tags, size_t ldz, uint64_t row0, cudaStream_t stream);
+                 const uint32_t* col_tags, size_t ldz, uint64_t row0, const uint32_t* col_tiles,
+                 const uint32_t* n_col_list, cudaStream_t stream);
 
 // Loads every form of the kernel on this device (once). Loading one may wait for the work on the device, so
 // contexts call this when they are made; without it the first launch does.

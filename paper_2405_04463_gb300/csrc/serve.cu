@@ -47,9 +47,10 @@ struct Variant {
   uint32_t tile_cols;
   int id;  // tcgen05: tile width; int8 paths: ring_gemm_i8_variant index
 };
-// The widths of listed column tiles. 256-column tiles run as two of 128, which the kernel computes at a
-// lower rate than 208-column ones; narrow tiles waste less on a few active columns. The first two can be
-// asked for by number, the others are the autotuner's.
+// The widths of listed column tiles. 256-column tiles run in the kernel with both operands in shared memory,
+// at a lower rate than 208-column ones (gemm_ts.cu) but with less waste just below a multiple of 256; narrow
+// tiles waste less on a few active columns. The first two can be asked for by number, the others are the
+// autotuner's.
 const Variant kTcVariants[] = {{"tc256", 256, 256}, {"tc128", 128, 128}, {"tc208", 208, 208}, {"tc64", 64, 64}};
 constexpr int kTcFixed = 2;
 const Variant kI8Variants[] = {{"mix128", 128, 0}, {"mma128", 128, 1}, {"mma64", 64, 2}, {"mma32", 32, 3}};
@@ -508,6 +509,8 @@ int autotune(Server& S) {
   const std::string key = tune_key(S);
   if (S.cfg.tune_cache && load_tuning(S, S.cfg.tune_cache, key)) return IPC_OK;
   const Chunk& ch = c->chunks[0];
+  int sms = 0;
+  SRV_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->cfg.device));
   cudaEvent_t e0, e1;
   SRV_TRY(cudaEventCreate(&e0));
   SRV_TRY(cudaEventCreate(&e1));
@@ -516,32 +519,44 @@ int autotune(Server& S) {
   std::vector<Bucket> b;
   bool first = true;
   // tcgen05: the narrow tiles are candidates while one of them, or two, cover the active columns (they
-  // compute at a lower rate), the wide ones above that
+  // compute at a lower rate), the wide ones above that; up to 64 columns one tile of 64 does
   const bool joint = tensor_path(S);
-  for (uint32_t cols = joint ? 64 : kPoolAlign; ; cols *= 2) {
+  std::vector<uint32_t> widths;
+  std::vector<bool> warm(S.n_variants, false);
+  if (joint) widths = {64, 128, 208, 256, 416};  // where one or two tiles of a width are full
+  for (uint32_t cols = joint ? 512 : kPoolAlign; widths.empty() || widths.back() < S.pool_pad; cols *= 2) widths.push_back(cols);
+  for (uint32_t cols : widths) {
     const uint32_t w = std::min(cols, S.pool_pad);
-    float best = 1e30f;
-    int best_v = 0;
-    std::ostringstream ms;
+    std::vector<int> candidates;
     for (int v = 0; v < S.n_variants; ++v) {
       const uint32_t tw = S.variants[v].tile_cols;
-      if (joint && (w <= 128) != (tw <= 128)) continue;
+      if (!joint || (w <= 64 ? tw == 64 : (w <= 128) == (tw <= 128))) candidates.push_back(v);
+    }
+    float best = 1e30f;
+    int best_v = candidates[0];
+    std::ostringstream ms;
+    for (size_t k = 0; k < candidates.size() && candidates.size() > 1; ++k) {
+      const int v = candidates[k];
+      const uint32_t tw = S.variants[v].tile_cols;
       std::vector<uint32_t> tiles((w + tw - 1) / tw);
-      for (uint32_t k = 0; k < tiles.size(); ++k) tiles[k] = k;
+      for (uint32_t t = 0; t < tiles.size(); ++t) tiles[t] = t;
       SRV_RC(upload_list(S, v, tiles, 0));
       SRV_TRY(cudaStreamSynchronize(c->sc));
-      // a pass as warm-up (which also sets the kernel attributes before any capture), then the passes that
-      // such a step launches together, two launches where it is one
-      const uint32_t per = joint ? launch_passes(S, v, ch, tiles.size()) : 1, reps = per > 1 ? 1 : 2;
+      // a pass as a variant's warm-up (which also sets its kernel's attributes before any capture), then as many
+      // as such a step launches together, three of them where they are many rounds of the chip
+      const bool many = tiles.size() * ((ch.rows + 127) / 128) >= 2.5 * sms;
+      const uint32_t n = joint ? std::min(launch_passes(S, v, ch, tiles.size()), many ? 3u : RING_GEMM_PASSES) : 1;
+      const uint32_t reps = n > 1 ? 1 : 2;
       auto launch = [&](uint32_t n) { return joint ? gemm_all(S, v, ch, n, n, c->sc) : gemm(S, v, ch, 0, 0, c->sc); };
-      SRV_RC(launch(1));
+      if (!warm[v]) SRV_RC(launch(1));
+      warm[v] = true;
       SRV_TRY(cudaEventRecord(e0, c->sc));
-      for (uint32_t rep = 0; rep < reps; ++rep) SRV_RC(launch(per));
+      for (uint32_t rep = 0; rep < reps; ++rep) SRV_RC(launch(n));
       SRV_TRY(cudaEventRecord(e1, c->sc));
       SRV_TRY(cudaEventSynchronize(e1));
       float t = 0;
       SRV_TRY(cudaEventElapsedTime(&t, e0, e1));
-      t /= static_cast<float>(reps * per);  // a pass
+      t /= static_cast<float>(reps * n);  // a pass
       ms << (ms.tellp() > 0 ? ", " : "") << "\"" << S.variants[v].name << "\": " << t;
       if (t < best) {
         best = t;
