@@ -178,8 +178,8 @@ def run_overlap(args, w):
 
 def run_fused(args, w):
     """The chunk step of a context, fused (one gemm_cmp_kernel launch per chunk: the six ring GEMMs
-    tile by tile and each tile's comparison phase, then the block join) and unfused (six GEMM
-    launches on the party streams and one comparison launch), on the workload's first --rows
+    tile by tile and each tile's comparison phase, then the block join) and unfused (GEMM
+    launches on one stream and one comparison launch), on the workload's first --rows
     database rows (one resident chunk for --rows <= 65,536), Galois-ring Shamir dots (--path tcg,
     the default) or replicated sharing (tc). Steps timed with CUDA events on the control stream."""
     import torch
@@ -486,8 +486,17 @@ def run_ours(args, w):
     hcode = [qcode[j].cpu().pin_memory() for j in range(3)]
     hmask = [qmask[j].cpu().pin_memory() for j in range(3)]
     torch.cuda.synchronize()
-    n_chunks = (w.s + 65535) // 65536
-    launches_per_step = 6 + n_chunks * 7 + 2
+    # query preparations; a chunk's GEMM launches (as ring_gemm_ts_passes groups them) and its comparison; the OR tree
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    cols = w.Q * w.R
+
+    def gemm_launches(chunk_rows):
+        rounds = -(-cols // 208) * -(-chunk_rows // 128) / sms
+        if 2 * 4 * 2 * w.l * cols <= 112 << 20 or 6 * rounds <= 32:
+            return 1
+        return 2 if 3 * rounds <= 32 else 6
+
+    launches_per_step = 6 + sum(gemm_launches(min(65536, w.s - r)) + 1 for r in range(0, w.s, 65536)) + 1
 
     def run_steps(ctx, k, host_inputs, gal=False, plain=False, lift=None, alternate=False):
         """k requests of the workload's query batch. Pipelined (default): up to the context's
@@ -679,8 +688,8 @@ def run_ours(args, w):
         "config": {"workload": w.name, "db_rows": w.s, "queries": w.Q, "rotations": w.R, "code_bits": w.l,
                    "planted": w.planted,
                    "path": "tc: int8 limbs as exact fp16 operands of tcgen05.mma (database resident as int8, "
-                           "widened in shared memory), fp32 TMEM accumulators re-based every 128 k inside "
-                           "[2^23, 2^24] (bit-exact; integer results; no rounding anywhere)",
+                           "widened into tensor memory), fp32 TMEM accumulators from 0, drained after at most "
+                           "1,024 products of at most 2^14 (bit-exact; integer results; no rounding anywhere)",
                    "parallelism": f"replicas x{world}",
                    "sharing": "3-party replicated (ABY3); galois_shamir_path: Galois-ring Shamir dots",
                    "l2": "inputs larger than L2: resident int8 limb planes 12 B x rows x 12800 = "

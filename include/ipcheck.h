@@ -231,12 +231,13 @@ int ipc_ring_gemm_tc(const int8_t* const x_lo[2], const int8_t* const x_hi[2], s
                      size_t ldz, uint64_t row0, void* stream);
 
 /*
- * IPC_PATH_TC with a tile width and an optional list of column tiles (the form the serving
- * loop replays inside a CUDA graph). tile_cols: 256 or 128 query columns per tile.
- * col_tiles (device, may be NULL): indices of the tiles of that width to compute, n_col_list
- * (device) their count, read when the kernel starts; with NULL every tile of [0, n_cols) is
- * computed, one CTA per tile. With a list the launch is persistent (one CTA per SM walking the
- * list), so its grid does not depend on the list. Other arguments and errors as ipc_ring_gemm_tc.
+ * IPC_PATH_TC with an optional list of column tiles (the form the serving loop replays inside a
+ * CUDA graph). tile_cols: 256 or 128, the query columns of a listed tile. col_tiles (device, may
+ * be NULL): indices of the tiles of that width to compute, n_col_list (device) their count, read
+ * when the kernel starts; the launch is persistent (one CTA per SM walking the list), so its grid
+ * does not depend on the list. With NULL every column of [0, n_cols) is computed as
+ * ipc_ring_gemm_tc does: tile_cols is checked and has no other effect, the library picks the tiles
+ * and may split K over the CTAs of a cluster. Other arguments and errors as ipc_ring_gemm_tc.
  */
 int ipc_ring_gemm_tc_tiles(uint32_t tile_cols, const int8_t* const x_lo[2], const int8_t* const x_hi[2],
                            size_t x_rows, const uint16_t* b_lo, const uint16_t* b_hi, uint32_t n_cols,
@@ -588,9 +589,10 @@ int ipc_check_persons(ipc_ctx* const ctx[2], const uint16_t* const code[6], cons
  * request loop on its own host thread. Requests (ipc_serve_submit) wait in FIFO order until
  * Q consecutive query slots of a column pool are free (admission by device memory: the pool
  * is allocated once, sized by pool_queries or from free device memory). One loop step runs
- * one resident chunk for every admitted column: the six GEMMs (A3) as one persistent launch
- * per party and vector over a device-side list of the column tiles in use, and the comparison
- * phase (A4-A8) over the same list, replayed from a CUDA graph per (chunk, GEMM variant). A
+ * one resident chunk for every admitted column: the six GEMMs (A3) as persistent launches over a
+ * device-side list of the column tiles in use (tcgen05 paths: one, two of three or six, by the
+ * columns in use; int8 paths: one per party and vector), and the comparison phase (A4-A8) over the
+ * same list, replayed from a CUDA graph per (chunk, GEMM variant, GEMMs of a launch). A
  * request visits every chunk once, starting wherever the loop is when it is admitted, then
  * its OR tree is finished (A8) and its slots freed. Its result does not depend on the other
  * requests: each PRF counter depends on its request id, query, rotation and row only.
@@ -602,7 +604,8 @@ int ipc_check_persons(ipc_ctx* const ctx[2], const uint16_t* const code[6], cons
 #define IPC_SERVE_AUTOTUNE -1
 typedef struct {
   uint32_t pool_queries;   /* query slots (R columns each); 0 = 2 x max_queries, or less if memory is short */
-  uint32_t max_pending;    /* submitted, not yet admitted requests before IPC_EAGAIN; 0 = 1024 */
+  uint32_t max_pending;    /* requests waiting for slots before IPC_EAGAIN; 0 = 1024. One that finds
+                              its slots free when it is submitted does not count */
   int32_t variant;         /* GEMM variant for every step, or IPC_SERVE_AUTOTUNE. IPC_PATH_TC:
                               0 = 256-column tcgen05 tiles, 1 = 128-column; int8 paths: the
                               IPC_GEMM_* variants */

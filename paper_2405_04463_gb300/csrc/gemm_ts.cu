@@ -732,8 +732,8 @@ uint32_t cdiv(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
 
 // Column tiles per row tile and the parts of K (a cluster's CTAs): the pair with the shortest estimate
 //     rounds of the chip x (k-blocks of a CTA x (250 + 2.45 tile columns) + a tile's start and end)
-// in cycles. The cost of a k-block is a line through launches of one tile per SM (330 cycles at 32 columns,
-// 410 at 64, 490 at 128, 600 at 160, 760 at 208). A few rounds count whole; over many, other launches and
+// in units of 0.55 ns. The cost of a k-block is a line through launches of whole rounds (181 ns at 32 columns,
+// 212 at 64, 315 at 128, 358 at 160, 415 at 208). A few rounds count whole; over many, other launches and
 // drifting tiles fill the last one.
 // At 1,000 rows x 4 columns splitting K by 8 gives 0.023 ms against 0.15 ms unsplit, at 1,000 x 279 0.042
 // against 0.085 ms with a guess of nine SMs in ten for clusters; 9,973 x 217 takes two tiles of 112 by 2
@@ -761,10 +761,10 @@ double pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t n_pass, uint32_t
 }
 
 // The estimate of the form with both operands in shared memory, whose tiles are 256 columns wide and take 1,030
-// of these cycles a k-block: less than two tiles of 128 (1,127), more than one of 208 and a part of the next
-// columns'. So it pays from 241 to 256 columns, and at 500 where it saves a round. A request of 248 columns,
-// sustained: 65,536 rows of Galois-ring shares 5.64 ms with tiles of 128 and 5.38 ms so, replicated 10.63 and
-// 10.27 ms; 8,000 x 496 Galois 1.41 and 1.36 ms. 4 % must be gained to leave the estimates' errors behind.
+// of these units a k-block (572 ns): less than two tiles of 128 (1,127). So it pays from 241 to 256 columns,
+// and around 500 where it saves a round. A request of 248 columns, sustained: 65,536 rows of Galois-ring shares
+// 5.64 ms with tiles of 128 and 5.42 ms so, replicated 10.63 and 10.34 ms; 8,000 x 496 Galois 1.41 and 1.36 ms.
+// 4 % must be gained to leave the estimates' errors behind.
 double ss_cost(uint32_t n_cols, uint32_t row_tiles, uint32_t n_pass, uint32_t kb_total, uint32_t sms) {
   const double rounds = static_cast<double>(n_pass) * cdiv(n_cols, 256) * row_tiles / sms;
   return (rounds < 8 ? std::ceil(rounds) : rounds + 0.5) * (1030.0 * kb_total + 10000) / 0.96;
