@@ -168,7 +168,7 @@ __global__ void prep_query32_kernel(const uint32_t* __restrict__ y, uint64_t pla
 // earlier form kept both operands in shared memory, drained every 64 k and needed two passes over K for
 // tiles of 256 columns, because four accumulators of that width do not fit the 512 TMEM columns; with A
 // in tensor memory narrow MMAs run at the same rate, and 96 columns leave room for two widened k-blocks.
-// 65,536 rows x 992 columns (K = 25,600): 21.6 ms against 22.7 ms; 30,000 x 496: 5.1 against 6.07 ms;
+// 65,536 rows x 992 columns (K = 25,600): 20.9 ms against 22.7 ms; 30,000 x 496: 5.06 against 6.07 ms;
 // 19,456 x 96 (a tile per SM): 0.59 against 1.60 ms; 1,000 x 31: 0.053 against 1.51 ms. Two warps that
 // issue, one for H and one for Lo, take 5.95 ms at 30,000 x 496.
 constexpr int TM = 128, KB = 32;
@@ -554,15 +554,23 @@ __global__ void __launch_bounds__(THREADS, 1)
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_rank));
   }
-  // the tile, nw columns wide: bands of up to 8 column tiles, all row tiles of a band before the next
+  // the tile, nw columns wide: the tiles with 16 columns more come first, and of each width bands of up to 8
+  // column tiles, all row tiles of a band before the next. A band's tiles stream K in step and share the
+  // database in L2; with both widths in a band they did not (65,536 x 992: 62.9 GB read for 25.3 so, 22.1 ms
+  // for 20.9; x 496 11.9 for 10.8).
   constexpr uint32_t kBand = 8;
   uint32_t q0, d0, nw;
   {
-    const uint32_t lin = blockIdx.x / n_rank;
-    const uint32_t band = lin / (kBand * p.n_rt), c0 = band * kBand;
-    const uint32_t width = p.n_ct - c0 < kBand ? p.n_ct - c0 : kBand;
-    const uint32_t in_band = lin - band * kBand * p.n_rt, ct = c0 + in_band % width;
     const uint32_t units = (p.n_cols + 15) / 16, base = units / p.n_ct, rem = units % p.n_ct;
+    uint32_t lin = blockIdx.x / n_rank, first = 0, of = rem;
+    if (lin >= rem * p.n_rt) {
+      lin -= rem * p.n_rt;
+      first = rem;
+      of = p.n_ct - rem;
+    }
+    const uint32_t band = lin / (kBand * p.n_rt), c0 = band * kBand;
+    const uint32_t width = of - c0 < kBand ? of - c0 : kBand;
+    const uint32_t in_band = lin - band * kBand * p.n_rt, ct = first + c0 + in_band % width;
     q0 = 16 * (ct * base + (ct < rem ? ct : rem));
     nw = 16 * (base + (ct < rem ? 1 : 0));
     d0 = in_band / width * TM;
@@ -612,7 +620,7 @@ cudaError_t ready() {
 // unequal ones fill half a round more than their number, but no round is shorter than the narrowest tile or
 // longer than the widest. `together` launches fill each other's last rounds. Then the parts of K, each with a
 // start and an end. Measured, tiles of two widths against equal ones with padding: 30,000 rows x 496 columns
-// 5.1-5.4 ms against 5.34-5.5, 17,000 x 372 2.14 against 2.38, 8,000 x 1,240 3.28 against 3.40.
+// 5.06 ms against 5.34, 17,000 x 372 2.14 against 2.38, 8,000 x 1,240 3.30 against 3.40.
 void pick_shape(uint32_t n_cols, uint32_t row_tiles, uint32_t kb_total, uint32_t together, uint32_t& n_ct, uint32_t& split) {
   int dev = 0;
   const uint32_t* at_once = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_at_once[dev] : nullptr;
@@ -666,13 +674,17 @@ int ring_gemm_tc32_ready() {
   return IPC_OK;
 }
 
-// Whether a chunk's Z_2^32 GEMMs run best one after another: where two of their query operands do not fit the
-// L2 together, unless a launch has so few rounds of the chip that their last ones weigh more. Requests of 30,000
-// rows x 496 columns without lifting, sustained: 32.0 ms on one stream, 33.8 ms on the party streams; 65,536 x
-// 992: 132 and 144 ms; 65,536 x 155 with ConstLift: 14.1 and 13.8 ms.
+// Whether a chunk's Z_2^32 GEMMs run best one after another: over many rounds of the chip three launches' tiles
+// drift until they no longer share what lies in L2, if that does not hold two query operands; over few, launches
+// side by side fill each other's last rounds. Requests without lifting, sustained, in ms (side by side / in turn):
+//     30,000 rows x   496 columns ( 9 rounds a launch)  29.6 /  30.5
+//     30,000      x   992         (17)                  59.6 /  59.5
+//     16,384      x 1,984         (18)                  66.2 /  63.6
+//     65,536      x   744         (27)                  99.7 /  96.4
+//     65,536      x   992         (37)                 129.9 / 125.9
 bool ring_gemm_tc32_in_turn(uint32_t segments, size_t x_rows, uint32_t n_cols, uint32_t l) {
   const double rounds = static_cast<double>(cdiv(n_cols, MAX_TN)) * cdiv(static_cast<uint32_t>(x_rows), TM) / sm_count_current();
-  return 2 * 8ull * segments * l * n_cols > L2_QUERY_BYTES && rounds >= 2;
+  return 2 * 8ull * segments * l * n_cols > L2_QUERY_BYTES && rounds >= 17;
 }
 
 // segments: 2 for K = 2l over [x[0..3] | x[4..7]] (ABY3 replicated sharing, x[4..7] the
