@@ -547,7 +547,7 @@ int autotune(Server& S) {
       const bool many = tiles.size() * ((ch.rows + 127) / 128) >= 2.5 * sms;
       const uint32_t n = joint ? std::min(launch_passes(S, v, ch, tiles.size()), many ? 3u : RING_GEMM_PASSES) : 1;
       const uint32_t reps = n > 1 ? 1 : 2;
-      auto launch = [&](uint32_t n) { return joint ? gemm_all(S, v, ch, n, n, c->sc) : gemm(S, v, ch, 0, 0, c->sc); };
+      auto launch = [&](uint32_t passes) { return joint ? gemm_all(S, v, ch, passes, passes, c->sc) : gemm(S, v, ch, 0, 0, c->sc); };
       if (!warm[v]) SRV_RC(launch(1));
       warm[v] = true;
       SRV_TRY(cudaEventRecord(e0, c->sc));
